@@ -394,7 +394,7 @@ int mdwf_force4d(mdwf_ctx *ctx, double *dSdU, double *S, const double *phi, int 
  * accumulators afterwards.
  */
 typedef struct {
-    char name[40];        /* e.g. "hop_gather_f32", "hop_dag_xpay_f16n", "m5_f64", "blas_f32" */
+    char name[40];        /* e.g. "hop_f32", "hop_dag_xpay_f16n", "m5_f64", "blas_f32" */
     long long launches;
     double ms;
     double bytes;

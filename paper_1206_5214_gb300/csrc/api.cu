@@ -7,10 +7,10 @@
 // with C the fifth-dimension shift (P- psi_{s+1} + P+ psi_{s-1}, mass -m on
 // the wrap-around), M+ = b5 (4 - M5) + 1, M- = c5 (4 - M5) - 1. Every s-mixing
 // factor is a real Ls x Ls matrix per chirality; A, K and their adjoints are
-// built here in FP64 by dense inversion of I. Two launches make one M:
-//   z_e  = K H_eo (M_phi psi_o)                  (gather fused into the hop)
+// built here in FP64 by dense inversion of I. Three launches make one M:
+//   z_e  = K H_eo w_o,  w_o = M_phi psi_o        (after a site-local pass)
 //   out  = psi_o - 1/4 A H_oe z_e                (xpay fused)
-// and three make M^dag = 1 - 1/4 M_phi^dag H'_oe K^dag H'_eo A^dag (H' the
+// and likewise M^dag = 1 - 1/4 M_phi^dag H'_oe K^dag H'_eo A^dag (H' the
 // hopping part of D_W^dag):
 //   v_o  = A^dag psi_o;  z_e = K^dag H'_eo v_o;  out = psi_o - 1/4 M_phi^dag H'_oe z_e.
 #include <math.h>
@@ -119,8 +119,7 @@ void replay_graph_counts(mdwf_ctx* c, long long replays) {
 }
 
 static void kernel_name(int kind, char* out, size_t n) {
-    static const char* base[KB_NUM] = {"hop", "hop_gather", "hop_xpay", "hop_gather_xpay", "hop_dag",
-                                       "hop_dag_xpay", "m5", "m5_xpay", "blas", "layout"};
+    static const char* base[KB_NUM] = {"hop", "hop_xpay", "hop_dag", "hop_dag_xpay", "m5", "m5_xpay", "blas", "layout"};
     static const char* prec[3] = {"f64", "f32", "f16n"};
     snprintf(out, n, "%s_%s", base[kind / 3], prec[kind % 3]);
 }
@@ -312,57 +311,50 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
 // ------------------------------------------------------------ operator chain
 
 int apply_op(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int dagger, int rhs0, const double* mask) {
-    const size_t fb = field_bytes(prec, c->g, nrhs);
+    int st;
+    if ((st = ensure_tmp(c, prec, nrhs))) return st;
+    return apply_chain(c, out, in, prec, nrhs, dagger, c->tmp[0].p, c->tmp[1].p,
+                       fx_exp_if(c, prec, c->tmp[0].p, nrhs), fx_exp_if(c, prec, c->tmp[1].p, nrhs),
+                       prec == MDWF_F64 ? (const void*)c->mass64 : (const void*)c->mass32, rhs0, mask);
+}
+
+int ensure_tmp(mdwf_ctx* c, int prec, int nrhs) {
+    const size_t bytes = prec == MDWF_F64 ? fx_field_bytes(c->g, nrhs) : field_bytes(prec, c->g, nrhs);
+    const int st = ensure_workspace(c->tmp[0], bytes);
+    return st ? st : ensure_workspace(c->tmp[1], bytes);
+}
+
+int to_fx(mdwf_ctx* c, void* dst, const void* src, int nrhs) {
+    M5Launch m{};
+    m.out = dst; m.in = src; m.coef = 1.0; m.nrhs = nrhs; m.sop = SOP_ID;
+    m.out_exp = fx_exponents(dst, c->g, nrhs);
+    return launch_m5(c, MDWF_F64, m);
+}
+
+int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int dagger, void* z, void* w, int* zexp,
+                int* wexp, const void* mass, int rhs0, const double* mask) {
     int st;
     note_apply(c, prec);
-    if ((st = ensure_workspace(c->tmp[0], fb))) return st;
-    if ((st = ensure_workspace(c->tmp[1], fb))) return st;
-    const void* mass = prec == MDWF_F64 ? (const void*)c->mass64 : (const void*)c->mass32;
-    HopLaunch h{};
-    h.nrhs = nrhs;
-    h.b5 = c->b5;
-    h.c5 = c->c5;
-    h.mass = mass;
-    h.mask = mask;
-    if (!dagger) {
-        // w_o = M_phi psi_o by one site-local pass, so that the first hop loads w
-        // without the gather along s (and the FP32 / FP16 hops can prefetch)
-        M5Launch m{};
-        m.out = c->tmp[1].p; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mask = mask;
-        set_sop(c, prec, SOP_MPHI, 0, m);
-        offset_rhs(c, prec, rhs0, m);
-        if ((st = launch_m5(c, prec, m))) return st;
-        // z_e = K H_eo w_o
-        h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.out_parity = 0;
-        h.gather = 0; h.dagger = 0;
-        set_sop(c, prec, SOP_K, 0, h);
-        offset_rhs(c, prec, rhs0, h);
-        if ((st = launch_hop(c, prec, h))) return st;
-        // out = psi_o - 1/4 A H_oe z_e
-        h.out = out; h.in = c->tmp[0].p; h.x = in; h.coef = -0.25; h.out_parity = 1;
-        h.gather = 0; h.dagger = 0;
-        h.mass = mass;
-        set_sop(c, prec, SOP_A, 0, h);
-        offset_rhs(c, prec, rhs0, h);
-        return launch_hop(c, prec, h);
-    }
-    // v_o = A^dag psi_o
+    // the first factor by a site-local pass: w_o = M_phi psi_o, or v_o = A^dag psi_o for M^dag
     M5Launch m{};
-    m.out = c->tmp[1].p; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mask = mask;
-    set_sop(c, prec, SOP_A, 1, m);
+    m.out = w; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mass = mass; m.mask = mask; m.out_exp = wexp;
+    set_sop(c, prec, dagger ? SOP_A : SOP_MPHI, dagger, m);
     offset_rhs(c, prec, rhs0, m);
     if ((st = launch_m5(c, prec, m))) return st;
-    // z_e = K^dag H'_eo v_o
-    h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.out_parity = 0;
-    h.gather = 0; h.dagger = 1;
-    set_sop(c, prec, SOP_K, 1, h);
+    HopLaunch h{};
+    h.nrhs = nrhs;
+    h.mask = mask;
+    h.dagger = dagger;
+    // z_e = K H_eo w_o, or K^dag H'_eo v_o
+    h.mass = mass;
+    h.out = z; h.in = w; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.in_exp = wexp; h.out_exp = zexp;
+    set_sop(c, prec, SOP_K, dagger, h);
     offset_rhs(c, prec, rhs0, h);
     if ((st = launch_hop(c, prec, h))) return st;
-    // out = psi_o - 1/4 M_phi^dag H'_oe z_e
-    h.out = out; h.in = c->tmp[0].p; h.x = in; h.coef = -0.25; h.out_parity = 1;
-    h.gather = 0; h.dagger = 1;
+    // out = psi_o - 1/4 A H_oe z_e, or psi_o - 1/4 M_phi^dag H'_oe z_e
     h.mass = mass;
-    set_sop(c, prec, SOP_MPHI, 1, h);
+    h.out = out; h.in = z; h.x = in; h.coef = -0.25; h.out_parity = 1; h.in_exp = zexp; h.out_exp = nullptr;
+    set_sop(c, prec, dagger ? SOP_MPHI : SOP_A, dagger, h);
     offset_rhs(c, prec, rhs0, h);
     return launch_hop(c, prec, h);
 }
@@ -527,6 +519,7 @@ int mdwf_destroy(mdwf_ctx* c) {
     cudaStreamSynchronize(c->stream);
     cudaGetLastError();  // an earlier call's failure was reported by that call
     for (int k = 0; k < 2; ++k) cudaFree(c->gauge[k]);
+    cudaFree(c->gauge_fx);
     cudaFree(c->tab64); cudaFree(c->tab32); cudaFree(c->mass64); cudaFree(c->mass32);
     cudaFreeHost(c->tab_host);
     cudaFree(c->tmp[0].p); cudaFree(c->tmp[1].p);
@@ -641,6 +634,12 @@ int mdwf_load_gauge(mdwf_ctx* c, const double* U, int where) {
         if (!c->gauge[k] && ((st = cuda_status(cudaMalloc(&c->gauge[k], bytes[k]))) ||
                              (st = canary_fill(c->gauge[k], bytes[k]))))
             return st;
+    if (!c->slab && !c->gauge_fx) {  // the fixed-point copy that the FP64 hops read
+        if ((st = cuda_status(cudaMalloc(&c->gauge_fx, nlink * (144 + sizeof(int))))) ||
+            (st = canary_fill(c->gauge_fx, nlink * (144 + sizeof(int)))))
+            return st;
+        c->gauge_fx_exp = (int*)((char*)c->gauge_fx + nlink * 144);
+    }
     const double* src = U;
     void* stage = nullptr;
     if (where == MDWF_HOST) {

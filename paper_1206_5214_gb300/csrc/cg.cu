@@ -25,6 +25,7 @@
 #include <cmath>
 #include <vector>
 
+#include "fx.cuh"
 #include "mdwf_internal.cuh"
 
 namespace mdwf {
@@ -114,7 +115,7 @@ template <int PX, int PR, int PP>
 __global__ void __launch_bounds__(128) k_pupd_w(Field<PX> x, Field<PR> r, Field<PP> p, Field<PP> w,
                                                const double* sc, const typename PrecTraits<PP>::real* mass,
                                                const typename PrecTraits<PP>::real* gs, Geom g, double b5,
-                                               double c5) {
+                                               double c5, int* wexp) {
     typedef typename PrecTraits<PX>::real RX;
     typedef typename PrecTraits<PR>::real RR;
     typedef typename PrecTraits<PP>::real RP;
@@ -166,7 +167,8 @@ __global__ void __launch_bounds__(128) k_pupd_w(Field<PX> x, Field<PR> r, Field<
     for (int k = 0; k < 12; ++k) wv[k] = bs * pv[k] + fm * row[sm * kRowStride + k];
 #pragma unroll
     for (int k = 12; k < 24; ++k) wv[k] = bs * pv[k] + fp * row[sp * kRowStride + k];
-    w.store(sr, s, wv);
+    if constexpr (PP == MDWF_F64) fx_store(w, wexp, sr, s, wv);  // the FP64 hops read fixed point
+    else w.store(sr, s, wv);
 }
 
 // dst = src (precision conversion); when sc != null only the right-hand sides
@@ -434,7 +436,8 @@ static int launch_pupd_w(Solver& S, void* x, void* r, void* p, void* w) {
     LaunchScope scope(c, KB_BLAS * 3 + PP, S.n5() * (3.0 * site_bytes(PR) + 3.0 * site_bytes(PP)), S.n5() * 144.0);
     if (cudaError_t e = launch_pdl(k_pupd_w<PR, PR, PP>, grid, block, smem, c->stream, make_field<PR>(x, S.g, S.nrhs),
                                    make_field<PR>(r, S.g, S.nrhs), make_field<PP>(p, S.g, S.nrhs),
-                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5, c->c5))
+                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5, c->c5,
+                                   fx_exp_if(c, PP, w, S.nrhs)))
         return cuda_status(e);
     return check_launch();
 }
@@ -445,6 +448,7 @@ template <int PP>
 static int init_w(Solver& S, void* w, const void* p, const double* mask = nullptr) {
     M5Launch m{};
     m.out = w; m.in = p; m.x = nullptr; m.coef = 1.0; m.nrhs = S.nrhs; m.mask = mask;
+    m.out_exp = fx_exp_if(S.c, PP, w, S.nrhs);
     set_sop(S.c, PP, SOP_MPHI, 0, m);
     return launch_m5(S.c, PP, m);
 }
@@ -466,14 +470,16 @@ static int cg_iteration_fused(Solver& S, void* x, void* r, void* p, void* t, voi
     const bool no_t = hop_no_t_ok(c, PP, S.nrhs);
     HopLaunch h{};
     h.nrhs = S.nrhs;
-    h.b5 = c->b5;
-    h.c5 = c->c5;
+    int* const zexp = fx_exp_if(c, PP, c->tmp[0].p, S.nrhs);
+    int* const vexp = fx_exp_if(c, PP, c->tmp[1].p, S.nrhs);
     h.mass = PP == MDWF_F64 ? (const void*)c->mass64 : (const void*)c->mass32;
     // z = K H_eo w, w = M_phi p (formed by the previous update)
-    h.out = c->tmp[0].p; h.in = w; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.gather = 0; h.dagger = 0;
+    h.out = c->tmp[0].p; h.in = w; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.dagger = 0;
+    h.in_exp = fx_exp_if(c, PP, w, S.nrhs); h.out_exp = zexp;
     set_sop(c, PP, SOP_K, 0, h);
     if ((st = launch_hop(c, PP, h))) return st;
-    h.out = t; h.in = c->tmp[0].p; h.x = p; h.coef = -0.25; h.out_parity = 1; h.gather = 0; h.dagger = 0;
+    h.out = t; h.in = c->tmp[0].p; h.x = p; h.coef = -0.25; h.out_parity = 1; h.dagger = 0;
+    h.in_exp = zexp; h.out_exp = vexp;
     set_sop(c, PP, SOP_A, 0, h);
     h.mat2 = nullptr;
     if (h.sop == SOP_DENSE) {  // the table of A^dag for v
@@ -487,11 +493,13 @@ static int cg_iteration_fused(Solver& S, void* x, void* r, void* p, void* t, voi
     h.no_t = 0;
     // K1' does not need alpha, so alpha is formed after it is launched, beside its end
     h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.dagger = 1;
+    h.in_exp = vexp; h.out_exp = zexp;
     set_sop(c, PP, SOP_K, 1, h);
     h.fuse = 0;
     if ((st = launch_hop(c, PP, h))) return st;
     if ((st = S.fin_hop(FIN_ALPHA, 1))) return st;
     h.out = c->tmp[1].p; h.in = c->tmp[0].p; h.x = no_t ? c->tmp[1].p : t; h.coef = -0.25; h.out_parity = 1;
+    h.in_exp = zexp; h.out_exp = nullptr;
     h.dagger = 1;
     set_sop(c, PP, SOP_MPHI, 1, h);
     h.fuse = 2; h.rfield = r; h.part = S.hpart; h.sc = S.sc; h.no_t = no_t;
@@ -923,7 +931,8 @@ static size_t solver_bytes(const mdwf_ctx* c, int nrhs, int inner, int nb, int h
     const size_t fpp = field_bytes(inner, c->g, nrhs);
     const int inner_fields = 3;
     return up256(f64) * 2 +
-           (inner == MDWF_F64 ? up256(f64) * inner_fields : up256(f32) * 2 + up256(fpp) * inner_fields) +
+           (inner == MDWF_F64 ? up256(f64) * (inner_fields - 1) + up256(fx_field_bytes(c->g, nrhs))
+                              : up256(f32) * 2 + up256(fpp) * inner_fields) +
            up256(sizeof(double) * S_NUM * kMaxRhs) + up256(sizeof(double) * nrhs * nb) +
            up256(sizeof(double) * nrhs * hb);
 }
@@ -989,7 +998,7 @@ static int solve_normal_mx(mdwf_ctx* c, int nrhs, void* xo, const void* src, con
     int ret = MDWF_OK;
     do {
         if ((st = ensure_workspace(c->solver, need))) { ret = st; break; }
-        if ((st = ensure_workspace(c->tmp[0], f64)) || (st = ensure_workspace(c->tmp[1], f64))) { ret = st; break; }
+        if ((st = ensure_tmp(c, MDWF_F64, nrhs))) { ret = st; break; }
         char* w = (char*)c->solver.p;
         auto take = [&](size_t bytes) { void* p = w; w += up(bytes); return p; };
         F.xo = xo;
@@ -998,7 +1007,7 @@ static int solve_normal_mx(mdwf_ctx* c, int nrhs, void* xo, const void* src, con
         const size_t fi = inner == MDWF_F64 ? f64 : fpp;
         if (inner != MDWF_F64) { F.xs = take(f32); F.rs = take(f32); }
         F.p = take(fi); F.t = take(fi);
-        F.w = take(fi);  // w = M_phi p
+        F.w = take(inner == MDWF_F64 ? fx_field_bytes(g, nrhs) : fi);  // w = M_phi p
         S.c = c; S.g = g; S.nrhs = nrhs; S.nb = nb;
         S.sc = (double*)take(sizeof(double) * S_NUM * kMaxRhs);
         S.part = (double*)take(sizeof(double) * nrhs * nb);
@@ -1078,8 +1087,7 @@ struct RhsScratch {
 
 // b_r -> (b_e, b'_o) with b'_o = A b_o + 1/2 A H_oe M_phi (A b_e), A = I^-1
 // (the Schur decomposition, D_br = -1/2 H_oe M_phi); xe and t are scratch.
-// M_phi A b_e = K b_e is formed by the site-local pass, so the hop needs no
-// gather along s.
+// M_phi A b_e = K b_e is formed by the site-local pass.
 int prepare_rhs(mdwf_ctx* c, const RhsScratch& w, const double* b, int where, int r) {
     const Geom& g = c->g;
     const size_t full1 = (size_t)g.Ls * 2 * g.Vh * 24 * sizeof(double);
@@ -1094,16 +1102,17 @@ int prepare_rhs(mdwf_ctx* c, const RhsScratch& w, const double* b, int where, in
     m.nrhs = 1; m.coef = 1.0; m.x = nullptr;
     set_sop(c, MDWF_F64, SOP_K, 0, m);
     offset_rhs(c, MDWF_F64, r, m);
-    m.out = w.xe; m.in = w.be;  // xe = K b_e = M_phi A b_e
+    m.out = w.xe; m.in = w.be;  // xe = K b_e = M_phi A b_e, in fixed point for the hop
+    m.out_exp = fx_exponents(w.xe, g, 1);
     if ((st = launch_m5(c, MDWF_F64, m))) return st;
-    m.mat = nullptr; m.mass = nullptr;
+    m.mat = nullptr; m.mass = nullptr; m.out_exp = nullptr;
     set_sop(c, MDWF_F64, SOP_A, 0, m);
     offset_rhs(c, MDWF_F64, r, m);
     m.out = w.t; m.in = w.bp;   // t = A b_o
     if ((st = launch_m5(c, MDWF_F64, m))) return st;
     HopLaunch h{};
-    h.nrhs = 1; h.b5 = c->b5; h.c5 = c->c5; h.mass = c->mass64;
-    h.out = w.bp; h.in = w.xe; h.x = w.t; h.coef = 0.5; h.out_parity = 1; h.gather = 0; h.dagger = 0;
+    h.nrhs = 1; h.mass = c->mass64;
+    h.out = w.bp; h.in = w.xe; h.in_exp = fx_exponents(w.xe, g, 1); h.x = w.t; h.coef = 0.5; h.out_parity = 1;
     set_sop(c, MDWF_F64, SOP_A, 0, h);
     offset_rhs(c, MDWF_F64, r, h);
     return launch_hop(c, MDWF_F64, h);
@@ -1132,14 +1141,15 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
     // staging of one full field). b_e and b'_o of every right-hand side are kept
     // from the preparation to the reconstruction when the device has room for
     // them; otherwise they are formed again from b after the solve.
-    const size_t lean = up(f64) * 2 + up(f1) * 4 + (where == MDWF_HOST ? up(full1) : 0);
-    const size_t keep_need = up(f64) * 4 + up(f1) * 2 + (where == MDWF_HOST ? up(full1) : 0);
+    const size_t fx1 = fx_field_bytes(g, 1);  // xe, the fixed-point input of the hops around the solve
+    const size_t lean = up(f64) * 2 + up(f1) * 3 + up(fx1) + (where == MDWF_HOST ? up(full1) : 0);
+    const size_t keep_need = up(f64) * 4 + up(f1) + up(fx1) + (where == MDWF_HOST ? up(full1) : 0);
     bool keep = true;
     {
         size_t free_b = 0, total_b = 0;
         if ((st = cuda_status(cudaMemGetInfo(&free_b, &total_b)))) return st;
         auto grow = [](size_t need_b, const Workspace& ws) { return need_b > ws.bytes ? need_b - ws.bytes : 0; };
-        size_t extra = grow(keep_need, c->io) + grow(f64, c->tmp[0]) + grow(f64, c->tmp[1]);
+        size_t extra = grow(keep_need, c->io) + grow(fx_field_bytes(g, nrhs), c->tmp[0]) + grow(fx_field_bytes(g, nrhs), c->tmp[1]);
         // the solver workspace, or the autotuner's two scratch fields before it (freed after tuning)
         size_t later = grow(
             solver_bytes(c, nrhs, prm.inner_prec, red_blocks(nrhs), hop_blocks(c, prm.inner_prec, nrhs)), c->solver);
@@ -1151,7 +1161,7 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
         keep = extra + (size_t(2) << 30) <= free_b;  // 2 GB left for the runtime and the caller
     }
     if ((st = ensure_workspace(c->io, keep ? keep_need : lean))) return st;
-    if ((st = ensure_workspace(c->tmp[0], f64)) || (st = ensure_workspace(c->tmp[1], f64))) return st;
+    if ((st = ensure_tmp(c, MDWF_F64, nrhs))) return st;
     char* w = (char*)c->io.p;
     auto take = [&](size_t bytes) { void* p = w; w += up(bytes); return p; };
     void *xo = take(f64), *src = take(f64);
@@ -1159,7 +1169,7 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
     void* bp_all = keep ? take(f64) : nullptr;
     RhsScratch sw;
     if (!keep) { sw.be = take(f1); sw.bp = take(f1); }
-    sw.xe = take(f1); sw.t = take(f1);
+    sw.xe = take(fx1); sw.t = take(f1);
     sw.stage = where == MDWF_HOST ? take(full1) : nullptr;
     auto point_at = [&](int r) {
         if (keep) { sw.be = (char*)be_all + (size_t)r * f1; sw.bp = (char*)bp_all + (size_t)r * f1; }
@@ -1196,13 +1206,14 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
         {
             M5Launch f{};  // xe (scratch until it is formed below) = M_phi x_o
             f.nrhs = 1; f.out = sw.xe; f.in = xo_r; f.x = nullptr; f.coef = 1.0;
+            f.out_exp = fx_exponents(sw.xe, g, 1);
             set_sop(c, MDWF_F64, SOP_MPHI, 0, f);
             offset_rhs(c, MDWF_F64, r, f);
             if ((st = launch_m5(c, MDWF_F64, f))) return st;
         }
         HopLaunch h{};  // t = 1/2 A H_eo M_phi x_o
-        h.nrhs = 1; h.b5 = c->b5; h.c5 = c->c5; h.mass = c->mass64;
-        h.out = sw.t; h.in = sw.xe; h.x = nullptr; h.coef = 0.5; h.out_parity = 0; h.gather = 0; h.dagger = 0;
+        h.nrhs = 1; h.mass = c->mass64;
+        h.out = sw.t; h.in = sw.xe; h.in_exp = fx_exponents(sw.xe, g, 1); h.x = nullptr; h.coef = 0.5; h.out_parity = 0;
         set_sop(c, MDWF_F64, SOP_A, 0, h);
         offset_rhs(c, MDWF_F64, r, h);
         if ((st = launch_hop(c, MDWF_F64, h))) return st;
@@ -1217,11 +1228,12 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
             void* z = c->tmp[0].p;
             M5Launch f{};
             f.nrhs = 1; f.out = z; f.in = sw.t; f.x = nullptr; f.coef = 2.0;
+            f.out_exp = fx_exponents(z, g, 1);
             set_sop(c, MDWF_F64, SOP_MPHI, 0, f);
             offset_rhs(c, MDWF_F64, r, f);
             if ((st = launch_m5(c, MDWF_F64, f))) return st;
             note_apply(c, MDWF_F64);
-            h.out = mx; h.in = z; h.x = xo_r; h.coef = -0.25; h.out_parity = 1; h.gather = 0; h.dagger = 0;
+            h.out = mx; h.in = z; h.in_exp = fx_exponents(z, g, 1); h.x = xo_r; h.coef = -0.25; h.out_parity = 1;
             h.mass = c->mass64;
             set_sop(c, MDWF_F64, SOP_A, 0, h);
             offset_rhs(c, MDWF_F64, r, h);

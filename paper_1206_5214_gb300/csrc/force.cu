@@ -180,7 +180,7 @@ extern "C" int mdwf_force(mdwf_ctx* c, double* dSdU, double* dSdb5, double* dSdc
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t need = up(f64) * 12 + (where == MDWF_HOST ? up(ub) + up(gb) : 0);
     if ((st = ensure_workspace(c->io, need))) return st;
-    if ((st = ensure_workspace(c->tmp[0], f64)) || (st = ensure_workspace(c->tmp[1], f64))) return st;
+    if ((st = ensure_tmp(c, MDWF_F64, 1))) return st;
     char* w = (char*)c->io.p;
     auto take = [&](size_t bytes) { void* p = w; w += up(bytes); return p; };
     void *ph = take(f64), *X = take(f64), *Y = take(f64), *al = take(f64), *de = take(f64), *h1 = take(f64);
@@ -215,23 +215,26 @@ extern "C" int mdwf_force(mdwf_ctx* c, double* dSdU, double* dSdb5, double* dSdc
     M5Launch m{};
     m.nrhs = 1; m.x = nullptr; m.coef = 1.0;
     HopLaunch h{};
-    h.nrhs = 1; h.b5 = c->b5; h.c5 = c->c5; h.mass = c->mass64; h.x = nullptr; h.coef = 1.0;
+    void* fx = c->tmp[1].p;  // the hops' fixed-point input
+    h.nrhs = 1; h.mass = c->mass64; h.x = nullptr; h.coef = 1.0; h.sop = SOP_ID;
+    h.in = fx; h.in_exp = fx_exponents(fx, g, 1);
     auto m5 = [&](void* out, const void* in, int sop, int swap, double coef, const void* x) {
         m.out = out; m.in = in; m.coef = coef; m.x = x;
         set_sop(c, MDWF_F64, sop, swap, m);
         return launch_m5(c, MDWF_F64, m);
     };
-    auto hop = [&](void* out, const void* in, int gather, int dagger) {
-        h.out = out; h.in = in; h.gather = gather; h.dagger = dagger; h.out_parity = 0; h.x = nullptr; h.coef = 1.0;
-        set_sop(c, MDWF_F64, SOP_ID, 0, h);
+    auto hop = [&](void* out, const void* in, int dagger) {  // H_eo in, or H'_eo in
+        const int e = to_fx(c, fx, in, 1);
+        if (e) return e;
+        h.out = out; h.dagger = dagger; h.out_parity = 0;
         return launch_hop(c, MDWF_F64, h);
     };
     if ((st = apply_op(c, Y, X, MDWF_F64, 1, 0))) return st;        // Y = M X
     if ((st = m5(al, Y, SOP_A, 1, 1.0, nullptr))) return st;         // alpha = A^dag Y
     if ((st = m5(de, X, SOP_MPHI, 0, 1.0, nullptr))) return st;      // delta = M_phi X
-    if ((st = hop(h1, X, 1, 0))) return st;                          // h1 = H_eo M_phi X
+    if ((st = hop(h1, de, 0))) return st;                            // h1 = H_eo delta
     if ((st = m5(be, h1, SOP_K, 0, 1.0, nullptr))) return st;        // beta = K h1
-    if ((st = hop(gp, al, 0, 1))) return st;                         // gamma' = H'_eo alpha
+    if ((st = hop(gp, al, 1))) return st;                         // gamma' = H'_eo alpha
     if ((st = m5(ga, gp, SOP_K, 1, 1.0, nullptr))) return st;        // gamma = K^dag gamma'
 
     if (dSdU) {
@@ -273,7 +276,7 @@ extern "C" int mdwf_force(mdwf_ctx* c, double* dSdU, double* dSdb5, double* dSdc
                 if ((st = slice_dot64(c, al, a1, r1.data()))) return st;
                 if ((st = slice_dot64(c, t3, a2, r2.data()))) return st;
             }
-            if ((st = hop(be, a3, 0, 0))) return st;  // H_eo X or H_eo C X
+            if ((st = hop(be, a3, 0))) return st;  // H_eo X or H_eo C X
             if ((st = slice_dot64(c, ga, be, r3.data()))) return st;
             for (int k = 0; k < Ls; ++k) dst[k] = 0.5 * (-4.0 * wgt * r1[k] + r2[k] + r3[k]);
         }
@@ -291,12 +294,12 @@ extern "C" int mdwf_force(mdwf_ctx* c, double* dSdU, double* dSdb5, double* dSdc
         if (which == 1 && (st = m5(t2, t2, SOP_C, 0, 1.0, nullptr))) return st;  // C v
         if ((st = m5(t3, t2, SOP_K, 0, -wgt, t2))) return st;           // (1 - w K) F v
         if ((st = field_dot64(c, gp, t3, 1, &r2))) return st;
-        const void* fx = X;
+        const void* fX = X;
         if (which == 1) {
             if ((st = m5(t1, X, SOP_C, 0, 1.0, nullptr))) return st;     // C X
-            fx = t1;
+            fX = t1;
         }
-        if ((st = hop(t2, fx, 0, 0))) return st;                         // H_eo F X
+        if ((st = hop(t2, fX, 0))) return st;                         // H_eo F X
         if ((st = field_dot64(c, ga, t2, 1, &r3))) return st;
         out[which] = 0.5 * (-4.0 * wgt * r1 + r2 + r3);
     }

@@ -1,0 +1,139 @@
+// Fixed-point form of the FP64 hopping operator's operands, and the hopping sum on it.
+//
+// Why: GB300 issues 2 FP64 FMAs per clock and SM (measured 2.1) but 64 32x32+64-bit integer
+// multiply-adds (measured 61). The hopping sum of one 5d site is about 770 FP64 operations, which bound
+// the FP64 operator at 1.8 ms per hop on 16^3 x 32 x 16 with the memory nearly idle. Done on 64-bit
+// integers it is 1728 multiply-adds of 32-bit limbs and a few thousand cheap integer operations: 0.50 to 0.59 ms
+// per hop (the FP64 s-operators of the epilogue are then over half of it), M^dag 3.92 -> 1.36 ms.
+//
+// Format: the 24 reals of one (site, s) spinor share a binary exponent e (the largest biased exponent
+// among them) and are stored as signed 64-bit integers q with value q 2^(e - 1080), |q| < 2^58. A link's
+// 18 reals share one in the same way, value u 2^(e - 1083), |u| < 2^61; they are stored as two signed
+// 32-bit limbs, u = hi 2^32 + lo.
+//
+// Error: a product drops lo x lo (below 2^62, a quarter of the last place of the sum) and the sum of a
+// term's six products is rounded to a multiple of 2^64, so a hopping sum is off by about one unit where
+// the largest of its eight neighbours' components, times a link entry of one, is 2^54 to 2^55 units.
+// FP64 arithmetic rounds every partial sum to 2^-53 of its size. M and M^dag against long double, 24 cases of
+// lattices, Ls, links and coefficients and four kinds of input (Gaussian, slices falling by e^-2, point
+// source, sites spread over decades): mean relative error 1.6e-16 in FP64, 1.3e-16 here; per site as well. Ranges: a neighbour's projected component is
+// below 2^59 (limbs |hi| <= 2^27, |lo| <= 2^31), so the middle sum is at most 6 (2^29 2^31 + 2^31 2^27) = 7.5
+// 2^60 < 2^63, a transported component at most 6 2^56, and the sum of eight terms at most 48 2^56 < 2^63.
+// Components more than 2^53 below the largest of their own spinor keep fewer bits than in FP64; each
+// is mixed with that component by the link and the spin projection that follow.
+//
+// Non-finite spinors are stored as the raw doubles with exponent kFxRaw, and a site that has such a
+// neighbour (or link) takes the FP64 arithmetic, so that infinities and NaN spread as there.
+#pragma once
+
+#include "mdwf_internal.cuh"
+
+namespace mdwf {
+
+template <int V> struct IntC { static constexpr int value = V; };
+
+constexpr int kFxFieldBias = 1080, kFxLinkBias = 1083;
+constexpr int kFxZero = -(1 << 20);   // exponent of an all-zero spinor or link
+constexpr int kFxRaw = 1 << 24;       // exponent of a spinor or link with a non-finite entry
+constexpr int kFxRawMin = 1 << 22;    // sums of exponents at or above this hold a kFxRaw
+
+// shared exponent of n doubles: the largest biased exponent, kFxZero or kFxRaw
+template <int N>
+__device__ __forceinline__ int fx_exponent(const double* v) {
+    int m = 0, low = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        m = max(m, __double2hiint(v[k]) & 0x7fffffff);
+        low |= __double2loint(v[k]);
+    }
+    const int e = m >> 20;
+    if (e == 0x7ff) return kFxRaw;
+    if (m == 0 && low == 0) return kFxZero;
+    return max(e, 1);  // subnormals carry the exponent 1
+}
+
+// v as an integer at the shared exponent e, with SH guard bits below the 53 of a double (truncated)
+template <int SH>
+__device__ __forceinline__ long long fx_mantissa(double v, int e) {
+    const int hi = __double2hiint(v);
+    const int ev = (hi >> 20) & 0x7ff;
+    const unsigned mh = (unsigned)(hi & 0xfffff) | (ev ? 0x100000u : 0u);
+    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(v)) << SH;
+    m >>= min(e - max(ev, 1), 63);
+    return hi < 0 ? -(long long)m : (long long)m;
+}
+
+__device__ __forceinline__ void fx_split(long long v, int& hi, int& lo) {
+    lo = (int)v;
+    hi = (int)((v + 0x80000000ll) >> 32);
+}
+
+// a 2^x as a double, rounded to nearest, by integer operations (the FP64 pipe would take a conversion and
+// a multiplication); x must keep the result a normal number (fx_scale_safe)
+__device__ __forceinline__ double fx_to_double(long long a, int x) {
+    const long long sgn = a >> 63;
+    const unsigned long long m0 = (unsigned long long)((a ^ sgn) - sgn);
+    const int lz = __clzll((long long)m0);
+    const unsigned long long m = m0 << (lz & 63);               // the top bit at 63
+    const unsigned long long rr = (m >> 11) + ((m >> 10) & 1);  // 53 bits, or 2^53 after a carry
+    const unsigned long long bits = ((unsigned long long)(unsigned)(1085 - lz + x) << 52) + rr;
+    const double d = __longlong_as_double((long long)(bits | ((unsigned long long)sgn << 63)));
+    return m0 == 0 ? 0.0 : d;
+}
+__device__ __forceinline__ bool fx_scale_safe(int x) { return x >= -1000 && x <= 950; }
+
+// Device view of a fixed-point field: the FP64 field's layout with integers, and [rhs][site][s] exponents.
+struct FxField {
+    const longlong2* v;
+    const int* e;
+    int Ls;
+    Bounds bnd;
+    __device__ __forceinline__ int exponent(long long sr, int s) const {
+        if (bnd.bad(sr, s, Ls)) return kFxZero;
+        return __ldg(e + sr * Ls + s);
+    }
+    __device__ __forceinline__ void load(long long sr, int s, long long* o) const {
+        if (bnd.bad(sr, s, Ls)) { for (int k = 0; k < 24; ++k) o[k] = 0; return; }
+        const longlong2* p = v + sr * 12 * Ls + s;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const longlong2 d = __ldg(p + (long long)k * Ls);
+            o[2 * k] = d.x;
+            o[2 * k + 1] = d.y;
+        }
+    }
+    // the spinor as doubles (the path of non-finite neighbours)
+    __device__ __forceinline__ void load(long long sr, int s, double* o) const {
+        long long q[24];
+        load(sr, s, q);
+        const int x = exponent(sr, s);
+        for (int k = 0; k < 24; ++k)
+            o[k] = x == kFxRaw ? __longlong_as_double(q[k]) : x == kFxZero ? 0.0 : scalbn((double)q[k], x - kFxFieldBias);
+    }
+};
+
+// writes a spinor of doubles in fixed point
+__device__ __forceinline__ void fx_store(const Field<MDWF_F64>& f, int* e, long long sr, int s, const double* v) {
+    if (f.bnd.bad(sr, s, f.Ls)) return;
+    const int x = fx_exponent<24>(v);
+    longlong2* p = reinterpret_cast<longlong2*>(f.v) + sr * 12 * f.Ls + s;
+    if (x == kFxRaw) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+            p[(long long)k * f.Ls] = make_longlong2(__double_as_longlong(v[2 * k]), __double_as_longlong(v[2 * k + 1]));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+            p[(long long)k * f.Ls] = make_longlong2(fx_mantissa<5>(v[2 * k], x), fx_mantissa<5>(v[2 * k + 1], x));
+    }
+    e[sr * f.Ls + s] = x;
+}
+
+// Fixed-point links: [link][9] of (re lo, re hi, im lo, im hi), and one exponent per link.
+struct FxGauge {
+    const int4* u;
+    const int* e;
+    Bounds bnd;
+};
+
+}  // namespace mdwf

@@ -36,18 +36,23 @@ static int solve_dag_dev(mdwf_ctx* c, double* x, const double* b, void* const* w
     if ((st = ensure_tables(c, 1, nullptr))) return st;
     if ((st = launch_split_full(c, be, bo, b, MDWF_F64, 1))) return st;
     M5Launch m;
-    m5_op(c, m, t, be, nullptr, 1.0, SOP_A, 1);  // t = I^-dag b_e
-    if ((st = launch_m5(c, MDWF_F64, m))) return st;
     HopLaunch h{};
-    h.nrhs = 1; h.b5 = c->b5; h.c5 = c->c5; h.mass = c->mass64;
-    h.out = bo; h.in = t; h.x = bo; h.coef = 0.5; h.out_parity = 1; h.gather = 0; h.dagger = 1;
-    set_sop(c, MDWF_F64, SOP_MPHI, 1, h);  // b'_o = b_o + 1/2 M_phi^dag H'_oe t
+    if ((st = ensure_tmp(c, MDWF_F64, 1))) return st;
+    void* fx = c->tmp[1].p;  // the hops' fixed-point input
+    h.nrhs = 1; h.mass = c->mass64;
+    h.in = fx; h.in_exp = fx_exponents(fx, c->g, 1);
+    h.out = bo; h.x = bo; h.coef = 0.5; h.out_parity = 1; h.dagger = 1;
+    set_sop(c, MDWF_F64, SOP_MPHI, 1, h);  // b'_o = b_o + 1/2 M_phi^dag H'_oe I^-dag b_e
+    m5_op(c, m, fx, be, nullptr, 1.0, SOP_A, 1);
+    m.out_exp = fx_exponents(fx, c->g, 1);
+    if ((st = launch_m5(c, MDWF_F64, m))) return st;
     if ((st = launch_hop(c, MDWF_F64, h))) return st;
     if ((st = solve_normal(c, 1, ww, bo, prm, res))) return st;
     if ((st = apply_op(c, y, ww, MDWF_F64, 1, 0))) return st;  // y = M w
     m5_op(c, m, xo, y, nullptr, 1.0, SOP_A, 1);                 // x_o = I^-dag y
     if ((st = launch_m5(c, MDWF_F64, m))) return st;
-    h.out = t; h.in = xo; h.x = be; h.coef = 0.5; h.out_parity = 0;
+    if ((st = to_fx(c, fx, xo, 1))) return st;
+    h.out = t; h.x = be; h.coef = 0.5; h.out_parity = 0;
     set_sop(c, MDWF_F64, SOP_MPHI, 1, h);  // t = b_e + 1/2 M_phi^dag H'_eo x_o
     if ((st = launch_hop(c, MDWF_F64, h))) return st;
     m5_op(c, m, be, t, nullptr, 1.0, SOP_A, 1);  // x_e = I^-dag t

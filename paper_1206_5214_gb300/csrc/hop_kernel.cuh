@@ -5,10 +5,8 @@
 //   out(x, s) = coef * sum_s' Mat_chi(s, s') [H w](x, s') (+ x_add(x, s))
 // where H is the Wilson hopping sum of Eq. (D^Wilson),
 //   H w(x) = sum_mu [(1 - g_mu) U_mu(x) w(x+mu) + (1 + g_mu) U_mu(x-mu)^dag w(x-mu)]
-// (projector signs flipped for the hopping part of D_W^dag), and w is either
-// the input field or the input with the fifth-dimension gather of Sec. 3
-// applied first: w_s = b5 psi_s + c5 (P+ psi_{s-1} + P- psi_{s+1}) with the
-// mass -m on the wrap-around terms (Eq. DWaction), i.e. w = M_phi psi.
+// (projector signs flipped for the hopping part of D_W^dag), and w is the input
+// field (M_phi psi, K H w, ..., formed by the kernel before).
 // Mat is an Ls x Ls real matrix per chirality (K = M_phi I^-1, I^-1, ...).
 //
 // Thread mapping: a block is Ls x SB threads: threadIdx.x = s, threadIdx.y =
@@ -23,10 +21,14 @@
 // applied after the hop through shared memory.
 #pragma once
 
+#include <math.h>
+
 #include <atomic>
 
-#include "mdwf_internal.cuh"
+#include "fx_hop.cuh"
 #include "mbarrier.cuh"
+#include "mdwf_internal.cuh"
+#include "spin.cuh"
 
 namespace mdwf {
 
@@ -36,13 +38,6 @@ template <typename R> struct HopParams {
                      // together share sites, so their links come from L2
     int out_parity;
     R coef;
-    // input gather w = gscale * (gown psi_s + gfac (P+ psi_{s-1} + P- psi_{s+1})) = M_phi psi;
-    // gscale is applied once to the accumulated hop instead of per neighbour
-    R gown, gfac, gscale;
-    // per-slice gather factors [gown(s)][gfac(s)][gscale(s)] (64 each) for
-    // s-dependent b5(s), c5(s), or null; gscale(s) then scales the hop of row s
-    // before the s-mixing and gscale above is 1
-    const R* gs;
     const R* mass;   // [rhs]
     const R* mat;    // dense tables [rhs][chir][s'][s] (sop == SOP_DENSE)
     const R* mat2;   // dense A^dag tables of the FUSE_T epilogue, same layout
@@ -90,140 +85,27 @@ __device__ __forceinline__ void halo_load(const HopParams<R>& hp, int dir, long 
     }
 }
 
-// --------------------------------------------------------- spin structure
-//
-// Chiral basis g_mu = [[0, A_mu], [A_mu^dag, 0]], A_k = -i sigma_k, A_4 = 1.
-// (1 + S g_mu) psi, psi = (u, l) by chirality halves, has upper half
-// h = u + S A l and lower half S A^dag h, so only h (2 spins x 3 colours) is
-// transported: project -> multiply by the link -> reconstruct.
-
-template <int MU, int S, typename R>
-__device__ __forceinline__ void project(const R* w, R* h) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const R u0r = w[2 * c], u0i = w[2 * c + 1], u1r = w[6 + 2 * c], u1i = w[7 + 2 * c];
-        const R l0r = w[12 + 2 * c], l0i = w[13 + 2 * c], l1r = w[18 + 2 * c], l1i = w[19 + 2 * c];
-        R a0r, a0i, a1r, a1i;  // (A l)_0, (A l)_1
-        if (MU == 0) {         // A = -i sigma_1: (A l)_0 = -i l1, (A l)_1 = -i l0
-            a0r = l1i; a0i = -l1r; a1r = l0i; a1i = -l0r;
-        } else if (MU == 1) {  // A = -i sigma_2: (A l)_0 = -l1, (A l)_1 = l0
-            a0r = -l1r; a0i = -l1i; a1r = l0r; a1i = l0i;
-        } else if (MU == 2) {  // A = -i sigma_3: (A l)_0 = -i l0, (A l)_1 = i l1
-            a0r = l0i; a0i = -l0r; a1r = -l1i; a1i = l1r;
-        } else {               // A = 1
-            a0r = l0r; a0i = l0i; a1r = l1r; a1i = l1i;
-        }
-        h[2 * c] = u0r + S * a0r;
-        h[2 * c + 1] = u0i + S * a0i;
-        h[6 + 2 * c] = u1r + S * a1r;
-        h[7 + 2 * c] = u1i + S * a1i;
-    }
-}
-
-// Transport and reconstruction of one hopping term: g[a][i] = sum_j V[i][j] h[a][j]
-// with V = U (or U^dag when ADJ; U row-major complex 3x3), then the upper half
-// of (1 + S g_mu) gets g and the lower half S A_mu^dag g. It runs one output
-// colour i at a time so that only one colour of g is live; `scaled` multiplies
-// g by `scale` first (the FP16 norm of the neighbour).
-template <bool ADJ, int MU, int S, typename R>
-__device__ __forceinline__ void transport_add(R* acc, const R* U, const R* h, R scale, bool scaled) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        R g[4];
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            // complex multiply-accumulate as four fused multiply-adds per term
-            R sr = 0, si = 0;
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const R ur = ADJ ? U[2 * (3 * j + i)] : U[2 * (3 * i + j)];
-                const R ui = ADJ ? -U[2 * (3 * j + i) + 1] : U[2 * (3 * i + j) + 1];
-                const R hr = h[6 * a + 2 * j], hi = h[6 * a + 2 * j + 1];
-                sr = fma(ur, hr, sr);
-                sr = fma(-ui, hi, sr);
-                si = fma(ur, hi, si);
-                si = fma(ui, hr, si);
-            }
-            g[2 * a] = scaled ? scale * sr : sr;
-            g[2 * a + 1] = scaled ? scale * si : si;
-        }
-        const R g0r = g[0], g0i = g[1], g1r = g[2], g1i = g[3];
-        acc[2 * i] += g0r;
-        acc[2 * i + 1] += g0i;
-        acc[6 + 2 * i] += g1r;
-        acc[7 + 2 * i] += g1i;
-        R b0r, b0i, b1r, b1i;  // (A^dag g)_0, (A^dag g)_1
-        if (MU == 0) {         // A^dag = i sigma_1: (i g1, i g0)
-            b0r = -g1i; b0i = g1r; b1r = -g0i; b1i = g0r;
-        } else if (MU == 1) {  // A^dag = i sigma_2: (g1, -g0)
-            b0r = g1r; b0i = g1i; b1r = -g0r; b1i = -g0i;
-        } else if (MU == 2) {  // A^dag = i sigma_3: (i g0, -i g1)
-            b0r = -g0i; b0i = g0r; b1r = g1i; b1i = -g1r;
-        } else {
-            b0r = g0r; b0i = g0i; b1r = g1r; b1i = g1i;
-        }
-        acc[12 + 2 * i] += S * b0r;
-        acc[13 + 2 * i] += S * b0i;
-        acc[18 + 2 * i] += S * b1r;
-        acc[19 + 2 * i] += S * b1i;
-    }
-}
-
-// Reconstruction alone, for a half spinor g already transported (the backward
-// t-direction term of a slab face, whose link lives on the sending slab):
-// upper half += f g, lower half += f S A_mu^dag g.
-template <int MU, int S, typename R>
-__device__ __forceinline__ void reconstruct_add(R* acc, const R* g, R f) {
-    static_assert(MU == 3, "slab faces are t-faces (A_4 = 1)");
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        acc[k] = fma(f, g[k], acc[k]);
-        acc[12 + k] = fma(S * f, g[k], acc[12 + k]);
-    }
-}
-
-// w = psi(s), or M_phi psi at s up to the factor gscale, for the neighbour column sr.
-// Returns a factor still to be applied to w (the FP16 norm of an ungathered
-// input, which is linear and is applied to the transported half spinor).
-template <int P, bool GATHER, typename R>
-__device__ __forceinline__ R load_input(const Field<P>& in, long long sr, int s, int Ls, R gown, R gfac,
-                                        R mass, R* w) {
-    if constexpr (P == MDWF_F16N && !GATHER) {
-        return in.load_raw(sr, s, w);
-    }
+// w = the neighbour spinor. Returns a factor still to be applied to w (the FP16 norm, which is linear and
+// is applied to the transported half spinor).
+template <typename IN, typename R>
+__device__ __forceinline__ R load_input(const IN& in, long long sr, int s, R* w) {
     in.load(sr, s, w);
-    if (GATHER) {
-        if (gown != R(1)) {
-#pragma unroll
-            for (int k = 0; k < 24; ++k) w[k] *= gown;
-        }
-        if (gfac != R(0)) {
-            R t[12];
-            const int sm = s > 0 ? s - 1 : Ls - 1;
-            const R fm = s > 0 ? gfac : -mass * gfac;
-            in.load_half(sr, sm, 0, t);  // P+ psi_{s-1}
-#pragma unroll
-            for (int k = 0; k < 12; ++k) w[k] += fm * t[k];
-            const int sp = s < Ls - 1 ? s + 1 : 0;
-            const R fp = s < Ls - 1 ? gfac : -mass * gfac;
-            in.load_half(sr, sp, 1, t);  // P- psi_{s+1}
-#pragma unroll
-            for (int k = 0; k < 12; ++k) w[12 + k] += fp * t[k];
-        }
-    }
     return R(1);
 }
+__device__ __forceinline__ float load_input(const Field<MDWF_F16N>& in, long long sr, int s, float* w) {
+    return in.load_raw(sr, s, w);
+}
 
-// The forward and backward terms of one direction mu together (FP64 operator,
-// no gather, no chemical potential on mu): per output colour i,
+// The forward and backward terms of one direction mu together (FP64 arithmetic,
+// no chemical potential on mu): per output colour i,
 //   g_f = [U_mu(x) h_f]_i,  s = g_f + [U_mu(x-mu)^dag h_b]_i  (one FMA chain from g_f),
 //   upper += s,  lower += SF A_mu^dag (g_f - g_b) with g_f - g_b = 2 g_f - s,
 // since the backward term enters the lower half with the opposite sign. This
 // takes 12 of the 48 additions of the two reconstructions away (the FP64
 // operator is bound by the FP64 pipe). Links are read one row (U) or one
 // column (U^dag) at a time.
-template <int MU, bool DAG>
-__device__ __forceinline__ void hop_pair64(double* acc, const Field<MDWF_F64>& in, const Gauge<MDWF_F64>& U,
+template <int MU, bool DAG, typename IN>
+__device__ __forceinline__ void hop_pair64(double* acc, const IN& in, const Gauge<MDWF_F64>& U,
                                            const HopParams<double>& hp, const int* nbi, long long site, int s,
                                            long long rbase) {
     constexpr int SF = DAG ? +1 : -1;
@@ -299,11 +181,10 @@ __device__ __forceinline__ void hop_pair64(double* acc, const Field<MDWF_F64>& i
 
 // nbi: the site's eight neighbour indices (x+mu, mu = 0..3, then x-mu), each
 // read just before its term so that none is held in a register across terms
-template <int P, int MU, bool GATHER, bool DAG, bool DD = false, typename R>
-__device__ __forceinline__ void hop_dir(R* acc, const Field<P>& in, const Gauge<P>& U, const HopParams<R>& hp,
-                                        const int* nbi, long long site, int s, long long rbase, R mass,
-                                        R gown, R gfac, int rhs = 0) {
-    if constexpr (P == MDWF_F64 && !GATHER) {
+template <int P, int MU, bool DAG, bool DD = false, typename IN, typename R>
+__device__ __forceinline__ void hop_dir(R* acc, const IN& in, const Gauge<P>& U, const HopParams<R>& hp,
+                                        const int* nbi, long long site, int s, long long rbase, int rhs = 0) {
+    if constexpr (P == MDWF_F64) {
         if (!(MU == 3 && (hp.chem || DD))) {
             hop_pair64<MU, DAG>(acc, in, U, hp, nbi, site, s, rbase);
             return;
@@ -311,7 +192,7 @@ __device__ __forceinline__ void hop_dir(R* acc, const Field<P>& in, const Gauge<
     }
     const Geom& g = hp.g;
     constexpr int SF = DAG ? +1 : -1;  // forward projector 1 + SF g_mu
-    constexpr bool SCALED = P == MDWF_F16N && !GATHER;
+    constexpr bool SCALED = P == MDWF_F16N;
     if constexpr (DD && MU == 3) {
         // slab faces: the neighbour across a face comes from the halo
         const int jf = __ldg(nbi + 3), jb = __ldg(nbi + 7);
@@ -332,7 +213,7 @@ __device__ __forceinline__ void hop_dir(R* acc, const Field<P>& in, const Gauge<
             const bool fwd = jb < 0;
             const long long j = fwd ? jf : jb;
             R w[24], h[12], u[18];
-            const R f = load_input<P, GATHER>(in, rbase + j, s, g.Ls, gown, gfac, mass, w);
+            const R f = load_input(in, rbase + j, s, w);
             if (fwd) {
                 project<3, SF>(w, h);
                 U.load(((long long)hp.out_parity * 4 + 3) * g.Vh + site, u);
@@ -348,7 +229,7 @@ __device__ __forceinline__ void hop_dir(R* acc, const Field<P>& in, const Gauge<
     {
         const long long jf = __ldg(nbi + MU);
         R w[24], h[12], u[18];
-        const R f = load_input<P, GATHER>(in, rbase + jf, s, g.Ls, gown, gfac, mass, w);
+        const R f = load_input(in, rbase + jf, s, w);
         project<MU, SF>(w, h);
         U.load(((long long)hp.out_parity * 4 + MU) * g.Vh + site, u);
         const bool tm = MU == 3 && hp.chem;
@@ -357,7 +238,7 @@ __device__ __forceinline__ void hop_dir(R* acc, const Field<P>& in, const Gauge<
     {
         const long long jb = __ldg(nbi + 4 + MU);
         R w[24], h[12], u[18];
-        const R f = load_input<P, GATHER>(in, rbase + jb, s, g.Ls, gown, gfac, mass, w);
+        const R f = load_input(in, rbase + jb, s, w);
         project<MU, -SF>(w, h);
         U.load(((long long)(1 - hp.out_parity) * 4 + MU) * g.Vh + jb, u);
         const bool tm = MU == 3 && hp.chem;
@@ -498,7 +379,7 @@ __device__ __forceinline__ void pf_term(R* acc, const Field<P>& in, const Gauge<
     constexpr int S = FWD ? SF : -SF;
     if constexpr (T < 7) {
         const long long jn = __ldg(nbi + TermOf<T + 1>::NB);
-        fnxt = load_input<P, false>(in, rbase + jn, s, hp.g.Ls, R(1), R(0), R(0), nxt);
+        fnxt = load_input(in, rbase + jn, s, nxt);
     }
     R h[12], u[18];
     project<MU, S>(cur, h);
@@ -517,7 +398,7 @@ __device__ __forceinline__ void hop_prefetch(R* acc, const Field<P>& in, const G
                                              const int* nbi, long long site, int s, long long rbase) {
     R wa[24], wb[24];
     R fa, fb = R(1);
-    fa = load_input<P, false>(in, rbase + __ldg(nbi + TermOf<0>::NB), s, hp.g.Ls, R(1), R(0), R(0), wa);
+    fa = load_input(in, rbase + __ldg(nbi + TermOf<0>::NB), s, wa);
     pf_term<P, 0, DAG>(acc, in, U, hp, nbi, site, s, rbase, wa, fa, wb, fb);
     pf_term<P, 1, DAG>(acc, in, U, hp, nbi, site, s, rbase, wb, fb, wa, fa);
     pf_term<P, 2, DAG>(acc, in, U, hp, nbi, site, s, rbase, wa, fa, wb, fb);
@@ -712,6 +593,36 @@ __device__ __forceinline__ void dense_columns(const R* mat, const R* col, int s,
 
 template <int P> struct ResPrec { static constexpr int value = P == MDWF_F64 ? MDWF_F64 : MDWF_F32; };
 
+// The FP64 operator's hops take fixed-point input (fx.cuh), except on t-slabs, whose halos are FP64.
+template <int P> struct FxArgs {};
+template <> struct FxArgs<MDWF_F64> : FxHop {};
+
+// The FP64 arithmetic for a site with a non-finite neighbour or link (rare: not inlined).
+template <bool DAG>
+__device__ __noinline__ void hop_nonfinite(double* acc, FxField in, Gauge<MDWF_F64> U, long long Vh, int out_parity,
+                                           bool chem, double efwd, double ebwd, const int* nbi, long long site, int s,
+                                           long long rbase) {
+    HopParams<double> hp;
+    hp.g.Vh = Vh; hp.out_parity = out_parity; hp.chem = chem; hp.efwd = efwd; hp.ebwd = ebwd;
+    for (int k = 0; k < 24; ++k) acc[k] = 0;
+    hop_dir<MDWF_F64, 0, DAG>(acc, in, U, hp, nbi, site, s, rbase);
+    hop_dir<MDWF_F64, 1, DAG>(acc, in, U, hp, nbi, site, s, rbase);
+    hop_dir<MDWF_F64, 2, DAG>(acc, in, U, hp, nbi, site, s, rbase);
+    hop_dir<MDWF_F64, 3, DAG>(acc, in, U, hp, nbi, site, s, rbase);
+}
+
+// a hop's result that the next hop reads: FP64 fields in fixed point where the launch says so
+template <int P, typename R>
+__device__ __forceinline__ void store_hop(const Field<P>& f, const FxArgs<P>& fx, long long sr, int s, const R* v) {
+    if constexpr (P == MDWF_F64) {
+        if (fx.out_exp) {
+            fx_store(f, fx.out_exp, sr, s, v);
+            return;
+        }
+    }
+    f.store(sr, s, v);
+}
+
 template <int P> struct FuseArgs {
     Field<P> out2;                     // FUSE_T: v = A^dag t
     Field<ResPrec<P>::value> rf;       // FUSE_R: residual r
@@ -765,14 +676,14 @@ constexpr bool kShuffleBidiag = MDWF_SHUFFLE_BIDIAG != 0;
 // launcher picks it when Ls matches), or -1 for the run-time choice; one
 // fixed length leaves the other lengths' code and its register demand out of
 // the kernel.
-template <int P, bool GATHER, bool DAG, bool XPAY, int FUSE, int STAGE, int LSR, bool DD = false>
+template <int P, bool DAG, bool XPAY, int FUSE, int STAGE, int LSR, bool DD = false>
 __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
                                       : STAGE == 3 ? kPrefetchMinBlocks
-                                                   : PrecTraits<P>::min_blocks - (GATHER ? 1 : 0))
+                                                   : PrecTraits<P>::min_blocks)
     hop_kernel(Field<P> out, Field<P> in, Field<P> xf, Gauge<P> U, HopParams<typename PrecTraits<P>::real> hp,
-               FuseArgs<P> fa) {
-    static_assert(!STAGE || (!GATHER && P != MDWF_F64), "staged loads: FP32 / FP16 operators without gather");
-    static_assert(!DD || (STAGE == 0 && !GATHER && FUSE == FUSE_NONE), "slab halos: plain loads, unfused");
+               FuseArgs<P> fa, FxArgs<P> fx) {
+    static_assert(!STAGE || P != MDWF_F64, "staged loads: FP32 / FP16 operators");
+    static_assert(!DD || (STAGE == 0 && FUSE == FUSE_NONE), "slab halos: plain loads, unfused");
     typedef typename PrecTraits<P>::real R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ls = hp.g.Ls;
@@ -798,12 +709,6 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     const bool active = site < hp.g.Vh;
     const long long rbase = (long long)rhs * hp.g.Vh;
     const R mass = hp.mass[rhs];
-    R gown = hp.gown, gfac = hp.gfac, gpre = R(1);
-    if (GATHER && hp.gs) {
-        gown = hp.gs[s];
-        gfac = hp.gs[64 + s];
-        gpre = hp.gs[128 + s];
-    }
     // the site's eight links into L1 before the terms need them (the links come from
     // L2, and a link load that waits for L2 inside a term stalls its chain): thread s
     // of the column asks for the lines of link s / 2 (forward links at the site,
@@ -841,7 +746,16 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         hop_bulk<P, DAG>(acc, in, U, hp, bk, bars, active, site, s, ly, tid, rbase);
     } else if (active) {
         const int4* nb = hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2;
-        if constexpr (STAGE == 3) {
+        if constexpr (P == MDWF_F64 && !DD) {
+            const int* nbi = reinterpret_cast<const int*>(nb);
+            if (!fx_hop<DAG>(acc, fx, hp.g, hp.out_parity, nbi, site, s, rbase)) {
+                double slow[24];
+                hop_nonfinite<DAG>(slow, fx.in, U, hp.g.Vh, hp.out_parity, hp.chem, hp.efwd, hp.ebwd, nbi, site, s,
+                                   rbase);
+#pragma unroll
+                for (int k = 0; k < 24; ++k) acc[k] = slow[k];
+            }
+        } else if constexpr (STAGE == 3) {
             hop_prefetch<P, DAG>(acc, in, U, hp, reinterpret_cast<const int*>(nb), site, s, rbase);
         } else if constexpr (STAGE == 1) {
             const int4 f = __ldg(nb), b = __ldg(nb + 1);
@@ -858,10 +772,10 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             hop_staged<P, DAG>(acc, in, U, hp, st, f, b, site, s, rbase);
         } else {
             const int* nbi = reinterpret_cast<const int*>(nb);
-            hop_dir<P, 0, GATHER, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, mass, gown, gfac, rhs);
-            hop_dir<P, 1, GATHER, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, mass, gown, gfac, rhs);
-            hop_dir<P, 2, GATHER, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, mass, gown, gfac, rhs);
-            hop_dir<P, 3, GATHER, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, mass, gown, gfac, rhs);
+            hop_dir<P, 0, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, rhs);
+            hop_dir<P, 1, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, rhs);
+            hop_dir<P, 2, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, rhs);
+            hop_dir<P, 3, DAG, DD>(acc, in, U, hp, nbi, site, s, rbase, rhs);
         }
     }
     if constexpr (STAGE == 1 || STAGE == 2) __syncthreads();
@@ -871,17 +785,13 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         if constexpr (XPAY) xf.prefetch(rbase + site, s);
         if constexpr (FUSE == FUSE_R) fa.rf.prefetch(rbase + site, s);
     }
-    if (GATHER && hp.gs) {
-#pragma unroll
-        for (int k = 0; k < 24; ++k) acc[k] *= gpre;
-    }
     if constexpr (FUSE == FUSE_T && XPAY && LSR == 16) {
         // t not stored (closed form, Ls = 16, two columns per warp): the rows go
         // to the column pass as y = cf acc + I p (I = M+ + M- C bidiagonal, by
         // shuffles), so that one pass forms t = A y = cf A acc + p, adds |t|^2
         // and turns t into v = A^dag t: one shared-memory round trip, not two
         if (hp.no_t && !dense && (blockDim.y & 1) == 0) {
-            const R cf = hp.coef * hp.gscale;
+            const R cf = hp.coef;
             R xv[24], y[24];
             if (active) {
                 xf.load(rbase + site, s, xv);
@@ -931,7 +841,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         }
     }
     if (FUSE == FUSE_NONE && !active) return;
-    const R cf = hp.coef * hp.gscale;
+    const R cf = hp.coef;
     bool xdone = false;
     if constexpr (XPAY && FUSE == FUSE_R && LSR == 16) {
         // x holds v = A^dag t: the addend t = I^dag v, I^dag = M+ + M- C^dag
@@ -962,7 +872,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         for (int k = 0; k < 24; ++k) res[k] *= cf;
     }
     if (FUSE == FUSE_NONE) {
-        out.store(rbase + site, s, res);
+        store_hop(out, fx, rbase + site, s, res);
         return;
     }
     R sq = 0;  // squared norm partial in the operator's arithmetic precision
@@ -982,13 +892,13 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         __syncthreads();
         if (dense) {
             dense_columns(mat2, hs + (size_t)ly * sst, s, Ls, res);
-            if (active) fa.out2.store(rbase + site, s, res);
+            if (active) store_hop(fa.out2, fx, rbase + site, s, res);
         } else {
             block_columns<LSR>(hs, blockDim.y, Ls, SOP_A, true, hp.sc, mass, tid, nthr);
             __syncthreads();
             if (active) {
                 row_load(mine, res);
-                fa.out2.store(rbase + site, s, res);
+                store_hop(fa.out2, fx, rbase + site, s, res);
             }
         }
     } else {  // FUSE_R
@@ -1012,7 +922,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 
 // ---------------------------------------------------------------- launcher
 
-template <int P, bool G, bool D, bool X, int FU, int ST, int LSR, bool DD = false>
+template <int P, bool D, bool X, int FU, int ST, int LSR, bool DD = false>
 static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<typename PrecTraits<P>::real>& hp) {
     typedef typename PrecTraits<P>::real R;
     const Geom& g = c->g;
@@ -1023,7 +933,7 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
                          : ST == 2 ? (size_t)2 * BulkBytes<P>::value * g.Ls * SB : 0;
     const int ntab = hp.sop == SOP_DENSE ? (FU == FUSE_T ? 2 : 1) : 0;
     size_t smem = kHopHeader + (size_t)ntab * 2 * g.Ls * g.Ls * sizeof(R) + (rows > stage ? rows : stage);
-    auto kern = hop_kernel<P, G, D, X, FU, ST, LSR, DD>;
+    auto kern = hop_kernel<P, D, X, FU, ST, LSR, DD>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_status(e);
@@ -1051,8 +961,7 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
     Gauge<P> U;
     U.u = reinterpret_cast<decltype(U.u)>(c->gauge[link_copy(P)]);
     U.bnd = make_bounds(8 * g.Vh);
-    const int base = D ? (X ? KB_HOP_DAG_XPAY : KB_HOP_DAG)
-                       : G ? (X ? KB_HOP_GATHER_XPAY : KB_HOP_GATHER) : (X ? KB_HOP_XPAY : KB_HOP);
+    const int base = D ? (X ? KB_HOP_DAG_XPAY : KB_HOP_DAG) : (X ? KB_HOP_XPAY : KB_HOP);
     const double n5 = (double)g.Vh * g.Ls * h.nrhs;
     // fields moved: in, out (+x), and for the fused epilogues v (FUSE_T) or r read+write instead of out (FUSE_R)
     const double sp = site_bytes(P), sr = site_bytes(ResPrec<P>::value);
@@ -1060,9 +969,25 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
     if (FU == FUSE_T && !hp.no_t) fields += sp;  // t (out) and v (out2); no_t stores only v
     if (FU == FUSE_R) fields += 2.0 * sr - sp;
     const double bytes = n5 * fields + 8.0 * g.Vh * link_bytes(P);
-    const double flops = n5 * (1320.0 + (G ? 72.0 : 0.0) + 144.0 + (X ? 48.0 : 0.0) + (FU ? 144.0 : 0.0));
+    const double flops = n5 * (1320.0 + 144.0 + (X ? 48.0 : 0.0) + (FU ? 144.0 : 0.0));
+    FxArgs<P> fx{};
+    if constexpr (P == MDWF_F64 && !DD) {
+        fx.in.v = reinterpret_cast<const longlong2*>(h.in);
+        fx.in.e = h.in_exp;
+        fx.in.Ls = g.Ls;
+        fx.in.bnd = in.bnd;
+        fx.U.u = reinterpret_cast<const int4*>(c->gauge_fx);
+        fx.U.e = c->gauge_fx_exp;
+        fx.U.bnd = U.bnd;
+        fx.out_exp = h.out_exp;
+        // e^{+-mu} = f 2^x, f in [1/2, 1)
+        const double f = frexp(hp.efwd, &fx.xf), b = frexp(hp.ebwd, &fx.xb);
+        fx.ff = hp.chem ? (long long)ldexp(f, 62) : 0;
+        fx.fb = hp.chem ? (long long)ldexp(b, 62) : 0;
+        if (!hp.chem) fx.xf = fx.xb = 0;
+    }
     LaunchScope scope(c, base * 3 + P, bytes, flops);
-    if (cudaError_t e = launch_pdl(kern, grid, block, smem, c->stream, out, in, xf, U, hp, fa)) return cuda_status(e);
+    if (cudaError_t e = launch_pdl(kern, grid, block, smem, c->stream, out, in, xf, U, hp, fa, fx)) return cuda_status(e);
     return check_launch();
 }
 
@@ -1070,27 +995,27 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
 // without the input gather have the staged variants; by default (mode 0, and
 // mode 3) they prefetch the next neighbour into registers. Mode 4 uses the
 // plain loads everywhere.
-template <int P, bool G, bool D, bool X, int FU>
+template <int P, bool D, bool X, int FU>
 static int launch_hop_pick(mdwf_ctx* c, const HopLaunch& h, const HopParams<typename PrecTraits<P>::real>& hp) {
-    if constexpr (!G && FU == FUSE_NONE && P != MDWF_F16N) {
-        if (h.halo) return launch_hop_variant<P, G, D, X, FU, 0, -1, true>(c, h, hp);
+    if constexpr (FU == FUSE_NONE && P != MDWF_F16N) {
+        if (h.halo) return launch_hop_variant<P, D, X, FU, 0, -1, true>(c, h, hp);
     }
     if (h.halo) return MDWF_EINVAL;
-    if constexpr (!G && P != MDWF_F64) {
+    if constexpr (P != MDWF_F64) {
         const int mode = c->hop_stage[P];
-        if (mode == 1) return launch_hop_variant<P, G, D, X, FU, 1, -1>(c, h, hp);
-        if (mode == 2) return launch_hop_variant<P, G, D, X, FU, 2, -1>(c, h, hp);
+        if (mode == 1) return launch_hop_variant<P, D, X, FU, 1, -1>(c, h, hp);
+        if (mode == 2) return launch_hop_variant<P, D, X, FU, 2, -1>(c, h, hp);
         if (mode == 3 || mode == 0) {
-            if (c->g.Ls == 16) return launch_hop_variant<P, G, D, X, FU, 3, 16>(c, h, hp);
-            return launch_hop_variant<P, G, D, X, FU, 3, -1>(c, h, hp);
+            if (c->g.Ls == 16) return launch_hop_variant<P, D, X, FU, 3, 16>(c, h, hp);
+            return launch_hop_variant<P, D, X, FU, 3, -1>(c, h, hp);
         }
     }
     // the FP32 / FP16 operators at Ls = 16 (the common length) with the
     // column length fixed at compile time
     if constexpr (P != MDWF_F64) {
-        if (c->g.Ls == 16) return launch_hop_variant<P, G, D, X, FU, 0, 16>(c, h, hp);
+        if (c->g.Ls == 16) return launch_hop_variant<P, D, X, FU, 0, 16>(c, h, hp);
     }
-    return launch_hop_variant<P, G, D, X, FU, 0, -1>(c, h, hp);
+    return launch_hop_variant<P, D, X, FU, 0, -1>(c, h, hp);
 }
 
 template <int P>
@@ -1101,19 +1026,6 @@ int launch_hop_t(mdwf_ctx* c, const HopLaunch& h) {
     hp.nrhs = h.nrhs;
     hp.out_parity = h.out_parity;
     hp.coef = (R)h.coef;
-    // M_phi = b5 + c5 C folded as b5 (1 + (c5/b5) C) when b5 != 0
-    if (h.b5 != 0.0) {
-        hp.gown = R(1); hp.gfac = (R)(h.c5 / h.b5); hp.gscale = (R)h.b5;
-    } else {
-        hp.gown = R(0); hp.gfac = (R)h.c5; hp.gscale = R(1);
-    }
-    if (!h.gather) { hp.gown = R(1); hp.gfac = R(0); hp.gscale = R(1); }
-    hp.gs = nullptr;
-    if (h.gather && c->sdep) {
-        hp.gown = R(1); hp.gfac = R(0); hp.gscale = R(1);
-        hp.gs = P == MDWF_F64 ? reinterpret_cast<const R*>(c->gs64) : reinterpret_cast<const R*>(c->gs32);
-        if (h.sop != SOP_DENSE || !hp.gs) return MDWF_EINVAL;
-    }
     hp.mass = reinterpret_cast<const R*>(h.mass);
     hp.mat = reinterpret_cast<const R*>(h.mat);
     hp.mat2 = reinterpret_cast<const R*>(h.mat2);
@@ -1139,6 +1051,9 @@ int launch_hop_t(mdwf_ctx* c, const HopLaunch& h) {
         set_error_message("a t-slab context applies its hops only through mdwf_slab_stage, with halos");
         return MDWF_EINVAL;
     }
+    // the FP64 hops read fixed-point fields; a t-slab's read and write FP64 ones
+    if (P == MDWF_F64 ? (h.in_exp == nullptr) != c->slab || (c->slab && h.out_exp) : h.in_exp || h.out_exp)
+        return MDWF_EINVAL;
     const bool X = h.x != nullptr;
     if (hp.no_t) {
         if (!hop_no_t_ok(c, P, h.nrhs) || h.fuse == FUSE_NONE || h.sop == SOP_DENSE) return MDWF_EINVAL;
@@ -1147,22 +1062,15 @@ int launch_hop_t(mdwf_ctx* c, const HopLaunch& h) {
     if (h.fuse != FUSE_NONE) {
         // fused CG epilogues: t = M p with v = A^dag t, or Ap = M^dag t folded into r
         // (structured s-operators or dense tables)
-        if (!X || h.gather || !h.part || !h.sc) return MDWF_EINVAL;
+        if (!X || !h.part || !h.sc) return MDWF_EINVAL;
         if (h.sop == SOP_DENSE && (!h.mat || (h.fuse == FUSE_T && !h.mat2))) return MDWF_EINVAL;
-        if (h.fuse == FUSE_T && !h.dagger && h.out2) return launch_hop_pick<P, false, false, true, FUSE_T>(c, h, hp);
-        if (h.fuse == FUSE_R && h.dagger && h.rfield) return launch_hop_pick<P, false, true, true, FUSE_R>(c, h, hp);
+        if (h.fuse == FUSE_T && !h.dagger && h.out2) return launch_hop_pick<P, false, true, FUSE_T>(c, h, hp);
+        if (h.fuse == FUSE_R && h.dagger && h.rfield) return launch_hop_pick<P, true, true, FUSE_R>(c, h, hp);
         return MDWF_EINVAL;
     }
-    if (h.gather) {
-        if (h.dagger) return MDWF_EINVAL;
-        return X ? launch_hop_pick<P, true, false, true, FUSE_NONE>(c, h, hp)
-                 : launch_hop_pick<P, true, false, false, FUSE_NONE>(c, h, hp);
-    }
     if (h.dagger)
-        return X ? launch_hop_pick<P, false, true, true, FUSE_NONE>(c, h, hp)
-                 : launch_hop_pick<P, false, true, false, FUSE_NONE>(c, h, hp);
-    return X ? launch_hop_pick<P, false, false, true, FUSE_NONE>(c, h, hp)
-             : launch_hop_pick<P, false, false, false, FUSE_NONE>(c, h, hp);
+        return X ? launch_hop_pick<P, true, true, FUSE_NONE>(c, h, hp) : launch_hop_pick<P, true, false, FUSE_NONE>(c, h, hp);
+    return X ? launch_hop_pick<P, false, true, FUSE_NONE>(c, h, hp) : launch_hop_pick<P, false, false, FUSE_NONE>(c, h, hp);
 }
 
 }  // namespace mdwf

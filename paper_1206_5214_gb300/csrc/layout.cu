@@ -1,5 +1,6 @@
 // Conversions between the user formats (complex128, lexicographic) and the
 // internal per-parity, s-innermost layouts of every precision.
+#include "fx.cuh"
 #include "mdwf_internal.cuh"
 
 namespace mdwf {
@@ -69,7 +70,9 @@ __global__ void full_kernel(Field<P> even, Field<P> odd, double* full, Geom g, i
     }
 }
 
-__global__ void gauge_pack_kernel(double2* u64, float* u32, const double2* __restrict__ U, Geom g) {
+// fx, fx_exp: the fixed-point copy (fx.cuh), or null
+__global__ void gauge_pack_kernel(double2* u64, float* u32, int4* fx, int* fx_exp, const double2* __restrict__ U,
+                                  Geom g) {
     const long long V = 2 * g.Vh;
     const long long n = V * 4;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -92,6 +95,25 @@ __global__ void gauge_pack_kernel(double2* u64, float* u32, const double2* __res
         }
         u32[l * 20 + 18] = 0.f;
         u32[l * 20 + 19] = 0.f;
+        if (fx) {
+            double v[18];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                v[2 * k] = src[k].x;
+                v[2 * k + 1] = src[k].y;
+            }
+            const int e = fx_exponent<18>(v);
+            fx_exp[l] = e;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                int4 o = make_int4(0, 0, 0, 0);
+                if (e != kFxRaw) {  // such a link is read from the FP64 copy
+                    fx_split(fx_mantissa<8>(v[2 * k], e), o.y, o.x);
+                    fx_split(fx_mantissa<8>(v[2 * k + 1], e), o.w, o.z);
+                }
+                fx[l * 9 + k] = o;
+            }
+        }
     }
 }
 
@@ -196,8 +218,9 @@ int launch_join_full(mdwf_ctx* c, double* full, const void* even, const void* od
 
 int launch_gauge_pack(mdwf_ctx* c, const double* U) {
     const long long n = 2 * c->g.Vh * 4;
-    LaunchScope scope(c, KB_LAYOUT * 3 + MDWF_F64, n * (144.0 * 2 + 80.0), 0.0);
+    LaunchScope scope(c, KB_LAYOUT * 3 + MDWF_F64, n * (144.0 * (c->gauge_fx ? 3 : 2) + 80.0), 0.0);
     gauge_pack_kernel<<<grid_for(n, 256), 256, 0, c->stream>>>((double2*)c->gauge[0], (float*)c->gauge[1],
+                                                                (int4*)c->gauge_fx, c->gauge_fx_exp,
                                                                 (const double2*)U, c->g);
     return check_launch();
 }

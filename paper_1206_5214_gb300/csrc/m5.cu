@@ -3,16 +3,29 @@
 // Sec. 3, M_phi, K = M_phi I^-1, the shift C, or a dense Ls x Ls table), or
 // their adjoints (chirality swapped). The Ls spinors of a 4d site are staged
 // in shared memory and each (site, component) column is solved by one thread.
+#include "fx.cuh"
 #include "mdwf_internal.cuh"
 
 namespace mdwf {
+
+// the result in its field, or in fixed point for the FP64 hops that read it
+template <int P, typename R>
+__device__ __forceinline__ void store_m5(const Field<P>& f, int* exp, long long sr, int s, const R* v) {
+    if constexpr (P == MDWF_F64) {
+        if (exp) {
+            fx_store(f, exp, sr, s, v);
+            return;
+        }
+    }
+    f.store(sr, s, v);
+}
 
 template <int P, bool XPAY>
 __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Field<P> xf,
                                                  const typename PrecTraits<P>::real* tab,
                                                  const typename PrecTraits<P>::real* mass,
                                                  typename PrecTraits<P>::real coef, Geom g, int sop, int swap,
-                                                 SCoef<typename PrecTraits<P>::real> sc, const double* mask) {
+                                                 SCoef<typename PrecTraits<P>::real> sc, const double* mask, int* out_exp) {
     typedef typename PrecTraits<P>::real R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ls = g.Ls;
@@ -63,7 +76,7 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
 #pragma unroll
             for (int k = 0; k < 24; ++k) v[k] += xv[k];
         }
-        out.store(sr, s, v);
+        store_m5(out, out_exp, sr, s, v);
         return;
     }
     if (dense) {
@@ -112,7 +125,7 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
 #pragma unroll
         for (int k = 0; k < 24; ++k) res[k] += xv[k];
     }
-    out.store(sr, s, res);
+    store_m5(out, out_exp, sr, s, res);
 }
 
 template <int P>
@@ -141,11 +154,13 @@ static int launch_m5_t(mdwf_ctx* c, const M5Launch& m) {
     if (m.x) {
         auto k = m5_kernel<P, true>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask);
+        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask,
+                                          m.out_exp);
     } else {
         auto k = m5_kernel<P, false>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask);
+        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask,
+                                          m.out_exp);
     }
     return check_launch();
 }

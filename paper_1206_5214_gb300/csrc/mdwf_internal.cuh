@@ -30,7 +30,7 @@
 // Blocks per SM the hop kernels are compiled for (register budget per thread:
 // 65536 / (128 * blocks)); overridable at build time.
 #ifndef MDWF_MINB_F64
-#define MDWF_MINB_F64 3
+#define MDWF_MINB_F64 4
 #endif
 #ifndef MDWF_MINB_F32
 #define MDWF_MINB_F32 8
@@ -130,6 +130,14 @@ inline size_t field_bytes(int prec, const Geom& g, int nrhs) {
         case MDWF_F16N: return n5 * 52;
     }
     return 0;
+}
+
+// A fixed-point FP64 field (fx.cuh): the FP64 field's bytes, then one int exponent per 5d site.
+inline size_t fx_field_bytes(const Geom& g, int nrhs) {
+    return field_bytes(MDWF_F64, g, nrhs) + (size_t)g.Vh * g.Ls * (size_t)nrhs * sizeof(int);
+}
+inline int* fx_exponents(void* field, const Geom& g, int nrhs) {
+    return (int*)((char*)field + field_bytes(MDWF_F64, g, nrhs));
 }
 
 // Cache hint: fetch the line of p into L1 (no register is written).
@@ -721,7 +729,7 @@ struct Workspace {
 
 // Kernel kinds for profiling and counting: kind = base * 3 + precision.
 enum KernelBase {
-    KB_HOP = 0, KB_HOP_GATHER, KB_HOP_XPAY, KB_HOP_GATHER_XPAY, KB_HOP_DAG, KB_HOP_DAG_XPAY,
+    KB_HOP = 0, KB_HOP_XPAY, KB_HOP_DAG, KB_HOP_DAG_XPAY,
     KB_M5, KB_M5_XPAY, KB_BLAS, KB_LAYOUT, KB_NUM
 };
 constexpr int KK_NUM = KB_NUM * 3;
@@ -749,6 +757,8 @@ struct mdwf_ctx {
     double M5 = 0, b5 = 0, c5 = 0, mf = 0;
     bool have_gauge = false;
     void* gauge[2] = {nullptr, nullptr};  // FP64 and FP32 copies
+    void* gauge_fx = nullptr;             // fixed-point copy (fx.cuh), 144 B per link as the FP64 one
+    int* gauge_fx_exp = nullptr;          // and its exponents, behind it in the same allocation
     // Ls x Ls tables for the current mass list, FP64 and FP32, plus per-rhs masses
     double* tab64 = nullptr;
     float* tab32 = nullptr;
@@ -872,15 +882,17 @@ struct HopLaunch {
     const void* x;        // xpay addend (same parity as out) or nullptr
     double coef;          // result = coef * Mat (H in) [+ x]
     int out_parity;
-    int gather;           // 1: apply M_phi (b5 + c5 C) to the input column before the hop
     int dagger;           // 1: hopping term of D_W^dag (projector signs flipped)
     const void* mat;      // dense table of the output Ls x Ls matrix (sop == SOP_DENSE), per rhs
     const void* mat2;     // dense table of A^dag for the FUSE_T epilogue (sop == SOP_DENSE)
     int sop;              // output s-operator (SOp)
     int swap;             // 1: the adjoint (chirality-swapped) s-operator
     const void* mass;     // per-rhs masses (double for F64, float otherwise)
-    double b5, c5;
     int nrhs;
+    // FP64 hops outside t-slabs read a fixed-point field (fx.cuh): its exponents (required), and, where the
+    // output (out, or out2 of fuse = 1) is to be fixed-point too, its exponents
+    const int* in_exp;
+    int* out_exp;
     const double* mask;   // per-rhs flags, or null: the blocks of a right-hand side whose flag is 0 do nothing
     // fused CG epilogues (0: none; 1: also v = A^dag out into out2 and |out|^2
     // partials; 2: r -= alpha out into rfield with |r|^2 partials, out not stored)
@@ -913,6 +925,7 @@ struct M5Launch {
     int swap;
     int nrhs;
     const void* mass; // per-rhs masses in this precision; nullptr = the context's
+    int* out_exp;     // FP64: write out in fixed point (fx.cuh) with these exponents
     const double* mask;  // per-rhs flags, or null (as HopLaunch::mask)
 };
 int launch_m5(mdwf_ctx* c, int prec, const M5Launch& m);
@@ -938,6 +951,17 @@ int launch_force(mdwf_ctx* c, double* dSdU, const void* A_odd, const void* B_eve
 // rhs0 + nrhs - 1 of the batch the tables were built for
 int apply_op(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int dagger, int rhs0 = 0,
              const double* mask = nullptr);
+// its launches on given intermediate fields z (even) and w (odd) and per-rhs masses; zexp, wexp: the exponents
+// of the FP64 operator's fixed-point intermediates (null for the other precisions)
+int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int dagger, void* z, void* w, int* zexp,
+                int* wexp, const void* mass, int rhs0, const double* mask);
+// the context's two intermediate fields at their size for (prec, nrhs)
+int ensure_tmp(mdwf_ctx* c, int prec, int nrhs);
+// dst (fx_field_bytes) = the FP64 field src in fixed point
+int to_fx(mdwf_ctx* c, void* dst, const void* src, int nrhs);
+inline int* fx_exp_if(const mdwf_ctx* c, int prec, void* field, int nrhs) {
+    return prec == MDWF_F64 ? fx_exponents(field, c->g, nrhs) : nullptr;
+}
 int tune_hop(mdwf_ctx* c, int prec, int nrhs, int* chosen);
 
 // solver (cg.cu)

@@ -29,12 +29,16 @@ constexpr size_t kNoAllocFieldBytes = (size_t)8 << 20;  // 8 MiB per intermediat
 constexpr int kNoAllocMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[2 * kNoAllocFieldBytes];
+// exponents of the two fields where they are fixed-point (the FP64 operator: 192 bytes a 5d site)
+constexpr size_t kNoAllocExps = kNoAllocFieldBytes / 192;
+static __device__ __align__(256) int g_noalloc_exp[2 * kNoAllocExps];
 static __device__ __align__(256) double g_noalloc_mass64[64];
 static __device__ __align__(256) float g_noalloc_mass32[64];
 
 struct NoAllocAddrs {
     bool ready = false;
     unsigned char* scratch = nullptr;
+    int *zexp = nullptr, *vexp = nullptr;
     double* mass64 = nullptr;
     float* mass32 = nullptr;
 };
@@ -51,6 +55,9 @@ static int noalloc_setup(int device, NoAllocAddrs** out) {
         int st;
         if ((st = cuda_status(cudaGetSymbolAddress(&p, g_noalloc_scratch)))) return st;
         a.scratch = (unsigned char*)p;
+        if ((st = cuda_status(cudaGetSymbolAddress(&p, g_noalloc_exp)))) return st;
+        a.zexp = (int*)p;
+        a.vexp = (int*)p + kNoAllocExps;
         if ((st = cuda_status(cudaGetSymbolAddress(&p, g_noalloc_mass64)))) return st;
         a.mass64 = (double*)p;
         if ((st = cuda_status(cudaGetSymbolAddress(&p, g_noalloc_mass32)))) return st;
@@ -138,32 +145,6 @@ extern "C" int mdwf_apply_noalloc(mdwf_ctx* c, void* out, const void* in, int pr
     void* z = a->scratch;
     void* v = a->scratch + kNoAllocFieldBytes;
     const void* mass = prec == MDWF_F64 ? (const void*)a->mass64 : (const void*)a->mass32;
-    note_apply(c, prec);
-    HopLaunch h{};
-    h.nrhs = nrhs;
-    h.b5 = c->b5;
-    h.c5 = c->c5;
-    h.mass = mass;
-    if (!dagger) {
-        M5Launch m{};  // v = M_phi psi (the first hop then needs no gather along s)
-        m.out = v; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mass = mass;
-        set_sop(c, prec, SOP_MPHI, 0, m);
-        if ((st = launch_m5(c, prec, m))) return st;
-        h.out = z; h.in = v; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.gather = 0; h.dagger = 0;
-        set_sop(c, prec, SOP_K, 0, h);
-        if ((st = launch_hop(c, prec, h))) return st;
-        h.out = out; h.in = z; h.x = in; h.coef = -0.25; h.out_parity = 1; h.gather = 0; h.dagger = 0;
-        set_sop(c, prec, SOP_A, 0, h);
-        return launch_hop(c, prec, h);
-    }
-    M5Launch m{};
-    m.out = v; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mass = mass;
-    set_sop(c, prec, SOP_A, 1, m);
-    if ((st = launch_m5(c, prec, m))) return st;
-    h.out = z; h.in = v; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.gather = 0; h.dagger = 1;
-    set_sop(c, prec, SOP_K, 1, h);
-    if ((st = launch_hop(c, prec, h))) return st;
-    h.out = out; h.in = z; h.x = in; h.coef = -0.25; h.out_parity = 1; h.gather = 0; h.dagger = 1;
-    set_sop(c, prec, SOP_MPHI, 1, h);
-    return launch_hop(c, prec, h);
+    return apply_chain(c, out, in, prec, nrhs, dagger != 0, z, v, prec == MDWF_F64 ? a->zexp : nullptr,
+                       prec == MDWF_F64 ? a->vexp : nullptr, mass, 0, nullptr);
 }

@@ -92,7 +92,8 @@ int apply_full_dev(mdwf_ctx* c, double* out, const double* in, int nrhs, int dag
     const size_t f64 = field_bytes(MDWF_F64, g, nrhs);
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     int st;
-    if ((st = ensure_workspace(c->aux, up(f64) * 4))) return st;
+    if ((st = ensure_workspace(c->aux, up(f64) * 4)) || (st = ensure_tmp(c, MDWF_F64, nrhs))) return st;
+    void* fx = c->tmp[1].p;
     char* w = (char*)c->aux.p;
     void *e = w, *o = w + up(f64), *oe = w + 2 * up(f64), *oo = w + 3 * up(f64);
     if ((st = launch_split_full(c, e, o, in, MDWF_F64, nrhs))) return st;
@@ -104,16 +105,15 @@ int apply_full_dev(mdwf_ctx* c, double* out, const double* in, int nrhs, int dag
         m.out = dst; m.in = same; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs;
         set_sop(c, MDWF_F64, SOP_MEE, dagger, m);
         if ((st = launch_m5(c, MDWF_F64, m))) return st;
+        // the hop's input in fixed point: M_phi of the other parity, or for D^dag that parity itself
+        m.out = fx; m.in = other; m.out_exp = fx_exponents(fx, g, nrhs);
+        if (!dagger) set_sop(c, MDWF_F64, SOP_MPHI, 0, m);
+        if ((st = dagger ? to_fx(c, fx, other, nrhs) : launch_m5(c, MDWF_F64, m))) return st;
         HopLaunch h{};
-        h.nrhs = nrhs; h.b5 = c->b5; h.c5 = c->c5; h.mass = c->mass64;
-        h.out = dst; h.in = other; h.x = dst; h.coef = -0.5; h.out_parity = par;
-        if (!dagger) {
-            h.gather = 1; h.dagger = 0;
-            set_sop(c, MDWF_F64, SOP_ID, 0, h);
-        } else {
-            h.gather = 0; h.dagger = 1;
-            set_sop(c, MDWF_F64, SOP_MPHI, 1, h);
-        }
+        h.nrhs = nrhs; h.mass = c->mass64; h.dagger = dagger;
+        h.out = dst; h.in = fx; h.in_exp = m.out_exp; h.x = dst; h.coef = -0.5; h.out_parity = par;
+        if (!dagger) h.sop = SOP_ID;
+        else set_sop(c, MDWF_F64, SOP_MPHI, 1, h);
         if ((st = launch_hop(c, MDWF_F64, h))) return st;
     }
     return launch_join_full(c, out, oe, oo, MDWF_F64, nrhs);

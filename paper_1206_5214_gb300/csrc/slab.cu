@@ -159,10 +159,7 @@ extern "C" int mdwf_slab_stage(mdwf_ctx* c, int stage, void* out, const void* in
     }
     HopLaunch h{};
     h.nrhs = nrhs;
-    h.b5 = c->b5;
-    h.c5 = c->c5;
     h.mass = mass;
-    h.gather = 0;
     h.dagger = dagger ? 1 : 0;
     h.halo = recv;
     if (stage == 1) {
