@@ -266,9 +266,9 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
         if ((st = cuda_status(cudaMalloc(&c->tab32, total * sizeof(float)))) ||
             (st = canary_fill(c->tab32, total * sizeof(float))))
             return st;
-        if ((st = cuda_status(cudaMalloc(&c->mass64, 64 * sizeof(double))))) return st;
-        if ((st = cuda_status(cudaMalloc(&c->mass32, 64 * sizeof(float))))) return st;
-        if ((st = cuda_status(cudaMallocHost(&c->tab_host, total * (sizeof(double) + sizeof(float)) + 64 * 12 + 16))))
+        if ((st = cuda_status(cudaMalloc(&c->mass64, 2 * kMaxRhs * sizeof(double))))) return st;
+        if ((st = cuda_status(cudaMalloc(&c->mass32, 2 * kMaxRhs * sizeof(float))))) return st;
+        if ((st = cuda_status(cudaMallocHost(&c->tab_host, total * (sizeof(double) + sizeof(float)) + 2 * kMaxRhs * 12 + 16))))
             return st;
         c->tab_cap = nrhs;
     }
@@ -276,7 +276,7 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
     double* h64 = c->tab_host;
     float* h32 = reinterpret_cast<float*>(h64 + total);
     double* hm64 = reinterpret_cast<double*>(h32 + total + (total & 1));
-    float* hm32 = reinterpret_cast<float*>(hm64 + 64);
+    float* hm32 = reinterpret_cast<float*>(hm64 + 2 * kMaxRhs);
     std::vector<double> one(per_rhs), b5s(Ls), c5s(Ls);
     for (int s = 0; s < Ls; ++s) {
         b5s[s] = c->sdep ? c->b5s[s] : c->b5;
@@ -291,15 +291,17 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
             memcpy(h64 + ((size_t)t * nrhs + r) * 2 * nn, one.data() + (size_t)t * 2 * nn, sizeof(double) * 2 * nn);
         hm64[r] = masses[r];
         hm32[r] = (float)masses[r];
+        hm64[kMaxRhs + r] = scoef_q(c, masses[r]);
+        hm32[kMaxRhs + r] = (float)hm64[kMaxRhs + r];
     }
     for (size_t i = 0; i < total; ++i) h32[i] = (float)h64[i];
     if ((st = cuda_status(cudaMemcpyAsync(c->tab64, h64, total * sizeof(double), cudaMemcpyHostToDevice, c->stream))))
         return st;
     if ((st = cuda_status(cudaMemcpyAsync(c->tab32, h32, total * sizeof(float), cudaMemcpyHostToDevice, c->stream))))
         return st;
-    if ((st = cuda_status(cudaMemcpyAsync(c->mass64, hm64, 64 * sizeof(double), cudaMemcpyHostToDevice, c->stream))))
+    if ((st = cuda_status(cudaMemcpyAsync(c->mass64, hm64, 2 * kMaxRhs * sizeof(double), cudaMemcpyHostToDevice, c->stream))))
         return st;
-    if ((st = cuda_status(cudaMemcpyAsync(c->mass32, hm32, 64 * sizeof(float), cudaMemcpyHostToDevice, c->stream))))
+    if ((st = cuda_status(cudaMemcpyAsync(c->mass32, hm32, 2 * kMaxRhs * sizeof(float), cudaMemcpyHostToDevice, c->stream))))
         return st;
     if ((st = cuda_status(cudaStreamSynchronize(c->stream)))) return st;
     memcpy(c->tab_masses, masses, sizeof(double) * nrhs);
@@ -338,6 +340,7 @@ int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int 
     // the first factor by a site-local pass: w_o = M_phi psi_o, or v_o = A^dag psi_o for M^dag
     M5Launch m{};
     m.out = w; m.in = in; m.x = nullptr; m.coef = 1.0; m.nrhs = nrhs; m.mass = mass; m.mask = mask; m.out_exp = wexp;
+    m.unscaled = 1;  // the factors of w and z go into the last launch's coefficient
     set_sop(c, prec, dagger ? SOP_A : SOP_MPHI, dagger, m);
     offset_rhs(c, prec, rhs0, m);
     if ((st = launch_m5(c, prec, m))) return st;
@@ -347,13 +350,14 @@ int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int 
     h.dagger = dagger;
     // z_e = K H_eo w_o, or K^dag H'_eo v_o
     h.mass = mass;
-    h.out = z; h.in = w; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.in_exp = wexp; h.out_exp = zexp;
+    h.out = z; h.in = w; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0; h.in_exp = wexp; h.out_exp = zexp;
     set_sop(c, prec, SOP_K, dagger, h);
     offset_rhs(c, prec, rhs0, h);
     if ((st = launch_hop(c, prec, h))) return st;
     // out = psi_o - 1/4 A H_oe z_e, or psi_o - 1/4 M_phi^dag H'_oe z_e
     h.mass = mass;
-    h.out = out; h.in = z; h.x = in; h.coef = -0.25; h.out_parity = 1; h.in_exp = zexp; h.out_exp = nullptr;
+    h.out = out; h.in = z; h.x = in; h.out_parity = 1; h.in_exp = zexp; h.out_exp = nullptr;
+    h.coef = -0.25 * ctx_scale(c, dagger ? SOP_A : SOP_MPHI) * ctx_scale(c, SOP_K); h.unscaled = 0;
     set_sop(c, prec, dagger ? SOP_MPHI : SOP_A, dagger, h);
     offset_rhs(c, prec, rhs0, h);
     return launch_hop(c, prec, h);

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const double* part, in
 // Column-blocked update for the fused iteration: block = (Ls, SB) threads
 // covering SB whole s-columns. x += alpha p; p = r + beta p; then
 // w = M_phi p = b5 p_s + c5 (P+ p_{s-1} + P- p_{s+1}) (mass -m on the
-// wrap-around) with the new p of the neighbouring slices taken from shared
+// wrap-around; without its factor b5 where the operators leave theirs out, sop_scale) with the new p of the neighbouring slices taken from shared
 // memory, so that the first hop of the next iteration reads w without
 // gathering along s. With per-slice coefficients gs holds the gather factors
 // of row s, [gown][gfac][gscale] (64 each): b5(s) = gscale gown and
@@ -164,9 +164,11 @@ __global__ void __launch_bounds__(128) k_pupd_w(Field<PX> x, Field<PR> r, Field<
     const RP fm = cs * (s > 0 ? RP(1) : -m), fp = cs * (s < Ls - 1 ? RP(1) : -m);
     RP wv[24];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) wv[k] = bs * pv[k] + fm * row[sm * kRowStride + k];
+    for (int k = 0; k < 24; ++k) wv[k] = bs == RP(1) ? pv[k] : bs * pv[k];
 #pragma unroll
-    for (int k = 12; k < 24; ++k) wv[k] = bs * pv[k] + fp * row[sp * kRowStride + k];
+    for (int k = 0; k < 12; ++k) wv[k] = fma(fm, row[sm * kRowStride + k], wv[k]);
+#pragma unroll
+    for (int k = 12; k < 24; ++k) wv[k] = fma(fp, row[sp * kRowStride + k], wv[k]);
     if constexpr (PP == MDWF_F64) fx_store(w, wexp, sr, s, wv);  // the FP64 hops read fixed point
     else w.store(sr, s, wv);
 }
@@ -433,21 +435,22 @@ static int launch_pupd_w(Solver& S, void* x, void* r, void* p, void* w) {
     const RP* mass = reinterpret_cast<const RP*>(PP == MDWF_F64 ? (const void*)c->mass64 : (const void*)c->mass32);
     const RP* gs = !c->sdep ? nullptr
                             : reinterpret_cast<const RP*>(PP == MDWF_F64 ? (const void*)c->gs64 : (const void*)c->gs32);
+    const double phi = ctx_scale(c, SOP_MPHI);  // w = M_phi p / phi
     LaunchScope scope(c, KB_BLAS * 3 + PP, S.n5() * (3.0 * site_bytes(PR) + 3.0 * site_bytes(PP)), S.n5() * 144.0);
     if (cudaError_t e = launch_pdl(k_pupd_w<PR, PR, PP>, grid, block, smem, c->stream, make_field<PR>(x, S.g, S.nrhs),
                                    make_field<PR>(r, S.g, S.nrhs), make_field<PP>(p, S.g, S.nrhs),
-                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5, c->c5,
+                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5 / phi, c->c5 / phi,
                                    fx_exp_if(c, PP, w, S.nrhs)))
         return cuda_status(e);
     return check_launch();
 }
 
-// w = M_phi p (the fused iteration's first hop reads w); with a mask, only the
+// w = M_phi p without its factor (the fused iteration's first hop reads w); with a mask, only the
 // right-hand sides whose entry is nonzero
 template <int PP>
 static int init_w(Solver& S, void* w, const void* p, const double* mask = nullptr) {
     M5Launch m{};
-    m.out = w; m.in = p; m.x = nullptr; m.coef = 1.0; m.nrhs = S.nrhs; m.mask = mask;
+    m.out = w; m.in = p; m.x = nullptr; m.coef = 1.0; m.unscaled = 1; m.nrhs = S.nrhs; m.mask = mask;
     m.out_exp = fx_exp_if(S.c, PP, w, S.nrhs);
     set_sop(S.c, PP, SOP_MPHI, 0, m);
     return launch_m5(S.c, PP, m);
@@ -473,12 +476,16 @@ static int cg_iteration_fused(Solver& S, void* x, void* r, void* p, void* t, voi
     int* const zexp = fx_exp_if(c, PP, c->tmp[0].p, S.nrhs);
     int* const vexp = fx_exp_if(c, PP, c->tmp[1].p, S.nrhs);
     h.mass = PP == MDWF_F64 ? (const void*)c->mass64 : (const void*)c->mass32;
-    // z = K H_eo w, w = M_phi p (formed by the previous update)
+    // z = K H_eo w, w = M_phi p (formed by the previous update). w, z and v go without the factors of their
+    // s-operators, which the coefficient of the second hop of M or M^dag takes instead
+    const double sk = ctx_scale(c, SOP_K);
+    h.unscaled = 1;
     h.out = c->tmp[0].p; h.in = w; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.dagger = 0;
     h.in_exp = fx_exp_if(c, PP, w, S.nrhs); h.out_exp = zexp;
     set_sop(c, PP, SOP_K, 0, h);
     if ((st = launch_hop(c, PP, h))) return st;
-    h.out = t; h.in = c->tmp[0].p; h.x = p; h.coef = -0.25; h.out_parity = 1; h.dagger = 0;
+    h.out = t; h.in = c->tmp[0].p; h.x = p; h.out_parity = 1; h.dagger = 0;
+    h.coef = -0.25 * ctx_scale(c, SOP_MPHI) * sk; h.unscaled = 0;
     h.in_exp = zexp; h.out_exp = vexp;
     set_sop(c, PP, SOP_A, 0, h);
     h.mat2 = nullptr;
@@ -492,13 +499,14 @@ static int cg_iteration_fused(Solver& S, void* x, void* r, void* p, void* t, voi
     h.mat2 = nullptr;
     h.no_t = 0;
     // K1' does not need alpha, so alpha is formed after it is launched, beside its end
-    h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.out_parity = 0; h.dagger = 1;
+    h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0; h.dagger = 1;
     h.in_exp = vexp; h.out_exp = zexp;
     set_sop(c, PP, SOP_K, 1, h);
     h.fuse = 0;
     if ((st = launch_hop(c, PP, h))) return st;
     if ((st = S.fin_hop(FIN_ALPHA, 1))) return st;
-    h.out = c->tmp[1].p; h.in = c->tmp[0].p; h.x = no_t ? c->tmp[1].p : t; h.coef = -0.25; h.out_parity = 1;
+    h.out = c->tmp[1].p; h.in = c->tmp[0].p; h.x = no_t ? c->tmp[1].p : t; h.out_parity = 1;
+    h.coef = -0.25 * ctx_scale(c, SOP_A) * sk; h.unscaled = 0;
     h.in_exp = zexp; h.out_exp = nullptr;
     h.dagger = 1;
     set_sop(c, PP, SOP_MPHI, 1, h);
@@ -1099,20 +1107,21 @@ int prepare_rhs(mdwf_ctx* c, const RhsScratch& w, const double* b, int where, in
     }
     if ((st = launch_split_full(c, w.be, w.bp, bdev, MDWF_F64, 1))) return st;
     M5Launch m{};
-    m.nrhs = 1; m.coef = 1.0; m.x = nullptr;
+    m.nrhs = 1; m.coef = 1.0; m.unscaled = 1; m.x = nullptr;
     set_sop(c, MDWF_F64, SOP_K, 0, m);
     offset_rhs(c, MDWF_F64, r, m);
     m.out = w.xe; m.in = w.be;  // xe = K b_e = M_phi A b_e, in fixed point for the hop
     m.out_exp = fx_exponents(w.xe, g, 1);
     if ((st = launch_m5(c, MDWF_F64, m))) return st;
-    m.mat = nullptr; m.mass = nullptr; m.out_exp = nullptr;
+    m.mat = nullptr; m.mass = nullptr; m.out_exp = nullptr; m.unscaled = 0;
     set_sop(c, MDWF_F64, SOP_A, 0, m);
     offset_rhs(c, MDWF_F64, r, m);
     m.out = w.t; m.in = w.bp;   // t = A b_o
     if ((st = launch_m5(c, MDWF_F64, m))) return st;
     HopLaunch h{};
     h.nrhs = 1; h.mass = c->mass64;
-    h.out = w.bp; h.in = w.xe; h.in_exp = fx_exponents(w.xe, g, 1); h.x = w.t; h.coef = 0.5; h.out_parity = 1;
+    h.out = w.bp; h.in = w.xe; h.in_exp = fx_exponents(w.xe, g, 1); h.x = w.t; h.out_parity = 1;
+    h.coef = 0.5 * ctx_scale(c, SOP_K);
     set_sop(c, MDWF_F64, SOP_A, 0, h);
     offset_rhs(c, MDWF_F64, r, h);
     return launch_hop(c, MDWF_F64, h);
@@ -1205,7 +1214,7 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
         if (!keep && (st = prepare_rhs(c, sw, b, where, r))) return st;  // b_e, b'_o again
         {
             M5Launch f{};  // xe (scratch until it is formed below) = M_phi x_o
-            f.nrhs = 1; f.out = sw.xe; f.in = xo_r; f.x = nullptr; f.coef = 1.0;
+            f.nrhs = 1; f.out = sw.xe; f.in = xo_r; f.x = nullptr; f.coef = 1.0; f.unscaled = 1;
             f.out_exp = fx_exponents(sw.xe, g, 1);
             set_sop(c, MDWF_F64, SOP_MPHI, 0, f);
             offset_rhs(c, MDWF_F64, r, f);
@@ -1213,7 +1222,8 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
         }
         HopLaunch h{};  // t = 1/2 A H_eo M_phi x_o
         h.nrhs = 1; h.mass = c->mass64;
-        h.out = sw.t; h.in = sw.xe; h.in_exp = fx_exponents(sw.xe, g, 1); h.x = nullptr; h.coef = 0.5; h.out_parity = 0;
+        h.out = sw.t; h.in = sw.xe; h.in_exp = fx_exponents(sw.xe, g, 1); h.x = nullptr; h.out_parity = 0;
+        h.coef = 0.5 * ctx_scale(c, SOP_MPHI);
         set_sop(c, MDWF_F64, SOP_A, 0, h);
         offset_rhs(c, MDWF_F64, r, h);
         if ((st = launch_hop(c, MDWF_F64, h))) return st;
@@ -1227,13 +1237,14 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
             // runs here
             void* z = c->tmp[0].p;
             M5Launch f{};
-            f.nrhs = 1; f.out = z; f.in = sw.t; f.x = nullptr; f.coef = 2.0;
+            f.nrhs = 1; f.out = z; f.in = sw.t; f.x = nullptr; f.coef = 1.0; f.unscaled = 1;
             f.out_exp = fx_exponents(z, g, 1);
             set_sop(c, MDWF_F64, SOP_MPHI, 0, f);
             offset_rhs(c, MDWF_F64, r, f);
             if ((st = launch_m5(c, MDWF_F64, f))) return st;
             note_apply(c, MDWF_F64);
-            h.out = mx; h.in = z; h.in_exp = fx_exponents(z, g, 1); h.x = xo_r; h.coef = -0.25; h.out_parity = 1;
+            h.out = mx; h.in = z; h.in_exp = fx_exponents(z, g, 1); h.x = xo_r; h.out_parity = 1;
+            h.coef = -0.5 * ctx_scale(c, SOP_MPHI);
             h.mass = c->mass64;
             set_sop(c, MDWF_F64, SOP_A, 0, h);
             offset_rhs(c, MDWF_F64, r, h);

@@ -562,16 +562,16 @@ enum { FUSE_NONE = 0, FUSE_T = 1, FUSE_R = 2 };
 template <typename R>
 __device__ __forceinline__ void bidiag_shuffle16(const R* in, R* out, int s, int op, bool swap, const SCoef<R>& sc,
                                                  R m) {
-    const R w0 = op == SOP_MPHI ? sc.b5 : op == SOP_MEE ? sc.Mp : R(0);
-    const R w1 = op == SOP_MPHI ? sc.c5 : op == SOP_MEE ? sc.Mm : R(1);
+    bool w0;
+    R w1;
+    bidiag_weights(op, sc, w0, w1);
     const int up = (s + 1) & 15, dn = (s + 15) & 15;
     const int src0 = swap ? up : dn, src1 = swap ? dn : up;
     const R f0 = w1 * ((swap ? s < 15 : s > 0) ? R(1) : -m);
     const R f1 = w1 * ((swap ? s > 0 : s < 15) ? R(1) : -m);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) out[k] = w0 * in[k] + f0 * __shfl_sync(0xffffffffu, in[k], src0, 16);
-#pragma unroll
-    for (int k = 12; k < 24; ++k) out[k] = w0 * in[k] + f1 * __shfl_sync(0xffffffffu, in[k], src1, 16);
+    for (int k = 0; k < 24; ++k)
+        out[k] = fma(k < 12 ? f0 : f1, __shfl_sync(0xffffffffu, in[k], k < 12 ? src0 : src1, 16), w0 ? in[k] : R(0));
 }
 
 // res = Mat col for the thread's slice s: Mat is the [chir][s'][s] table of one
@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     const bool active = site < hp.g.Vh;
     const long long rbase = (long long)rhs * hp.g.Vh;
     const R mass = hp.mass[rhs];
+    const SMass<R> sm{mass, hp.mass[kMaxRhs + rhs]};
     // the site's eight links into L1 before the terms need them (the links come from
     // L2, and a link load that waits for L2 inside a term stalls its chain): thread s
     // of the column asks for the lines of link s / 2 (forward links at the site,
@@ -787,9 +788,9 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     }
     if constexpr (FUSE == FUSE_T && XPAY && LSR == 16) {
         // t not stored (closed form, Ls = 16, two columns per warp): the rows go
-        // to the column pass as y = cf acc + I p (I = M+ + M- C bidiagonal, by
-        // shuffles), so that one pass forms t = A y = cf A acc + p, adds |t|^2
-        // and turns t into v = A^dag t: one shared-memory round trip, not two
+        // to the column pass as y = cf acc + (1 + r C) p (bidiagonal, by shuffles;
+        // cf holds 1 / M+), so that one pass forms t = A~ y = A (..) + p, adds |t|^2
+        // and turns t into A~^dag t: one shared-memory round trip, not two
         if (hp.no_t && !dense && (blockDim.y & 1) == 0) {
             const R cf = hp.coef;
             R xv[24], y[24];
@@ -805,7 +806,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             R* row = hs + (size_t)ly * site_stride(16) + s * kRowStride;
             row_store(row, y);
             __syncthreads();
-            const R sq = block_columns_a_adag<16>(hs, blockDim.y, hp.sc, mass, tid, nthr);
+            const R sq = block_columns_a_adag<16>(hs, blockDim.y, hp.sc, sm, tid, nthr);
             __syncthreads();
             if (active) {
                 row_load(row, y);
@@ -829,13 +830,18 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             shuffled = true;
         }
     }
+    if (!dense && hp.sop == SOP_ID) {
+#pragma unroll
+        for (int k = 0; k < 24; ++k) res[k] = acc[k];
+        shuffled = true;
+    }
     if (!shuffled) {
         row_store(mine, acc);
         __syncthreads();
         if (dense) {
             dense_columns(mat, hs + (size_t)ly * sst, s, Ls, res);
         } else {
-            block_columns<LSR>(hs, blockDim.y, Ls, hp.sop, hp.swap != 0, hp.sc, mass, tid, nthr);
+            block_columns<LSR>(hs, blockDim.y, Ls, hp.sop, hp.swap != 0, hp.sc, sm, tid, nthr);
             __syncthreads();
             row_load(mine, res);
         }
@@ -844,7 +850,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     const R cf = hp.coef;
     bool xdone = false;
     if constexpr (XPAY && FUSE == FUSE_R && LSR == 16) {
-        // x holds v = A^dag t: the addend t = I^dag v, I^dag = M+ + M- C^dag
+        // x holds M+ v = A~^dag t: the addend t = I^dag v = (1 + r C^dag) x
         // bidiagonal, by shuffles (every lane takes part; the launcher admits
         // no_t only where the shuffled s-operators run)
         if (hp.no_t) {
@@ -867,7 +873,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         xf.load(rbase + site, s, xv);
 #pragma unroll
         for (int k = 0; k < 24; ++k) res[k] = fma(cf, res[k], xv[k]);
-    } else {
+    } else if (cf != R(1)) {
 #pragma unroll
         for (int k = 0; k < 24; ++k) res[k] *= cf;
     }
@@ -894,7 +900,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             dense_columns(mat2, hs + (size_t)ly * sst, s, Ls, res);
             if (active) store_hop(fa.out2, fx, rbase + site, s, res);
         } else {
-            block_columns<LSR>(hs, blockDim.y, Ls, SOP_A, true, hp.sc, mass, tid, nthr);
+            block_columns<LSR>(hs, blockDim.y, Ls, SOP_A, true, hp.sc, sm, tid, nthr);
             __syncthreads();
             if (active) {
                 row_load(mine, res);
@@ -1025,17 +1031,14 @@ int launch_hop_t(mdwf_ctx* c, const HopLaunch& h) {
     hp.g = c->g;
     hp.nrhs = h.nrhs;
     hp.out_parity = h.out_parity;
-    hp.coef = (R)h.coef;
+    hp.coef = (R)(h.unscaled ? h.coef : h.coef * sop_scale(c, h.sop));
     hp.mass = reinterpret_cast<const R*>(h.mass);
     hp.mat = reinterpret_cast<const R*>(h.mat);
     hp.mat2 = reinterpret_cast<const R*>(h.mat2);
     hp.nbr = reinterpret_cast<const int4*>(c->nbr);
     hp.sop = h.sop;
     hp.swap = h.swap;
-    hp.sc.b5 = (R)c->b5;
-    hp.sc.c5 = (R)c->c5;
-    hp.sc.Mp = (R)(c->b5 * (4.0 - c->M5) + 1.0);
-    hp.sc.Mm = (R)(c->c5 * (4.0 - c->M5) - 1.0);
+    hp.sc = make_scoef<R>(c);
     // the adjoint's hopping matrix is transposed: the two factors exchange
     hp.chem = c->chem != 0.0;
     hp.efwd = (R)exp(h.dagger ? -c->chem : c->chem);

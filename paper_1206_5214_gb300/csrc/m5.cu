@@ -52,8 +52,9 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
         R v[24];
         in.load(sr, s, v);
         if (bidiag) {
-            const R w0 = sop == SOP_MPHI ? sc.b5 : sop == SOP_MEE ? sc.Mp : R(0);
-            const R w1 = sop == SOP_MPHI ? sc.c5 : sop == SOP_MEE ? sc.Mm : R(1);
+            bool w0;
+            R w1;
+            bidiag_weights(sop, sc, w0, w1);
             const R m = mass[rhs];
             const bool sw = swap != 0;
             const int up = s + 1 < Ls ? s + 1 : 0, dn = s > 0 ? s - 1 : Ls - 1;
@@ -64,17 +65,18 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
             in.load_half(sr, sw ? dn : up, 1, h1);
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
-                v[k] = w0 * v[k] + f0 * h0[k];
-                v[12 + k] = w0 * v[12 + k] + f1 * h1[k];
+                v[k] = fma(f0, h0[k], w0 ? v[k] : R(0));
+                v[12 + k] = fma(f1, h1[k], w0 ? v[12 + k] : R(0));
             }
         }
-#pragma unroll
-        for (int k = 0; k < 24; ++k) v[k] *= coef;
         if (XPAY) {
             R xv[24];
             xf.load(sr, s, xv);
 #pragma unroll
-            for (int k = 0; k < 24; ++k) v[k] += xv[k];
+            for (int k = 0; k < 24; ++k) v[k] = fma(coef, v[k], xv[k]);
+        } else if (coef != R(1)) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k) v[k] *= coef;
         }
         store_m5(out, out_exp, sr, s, v);
         return;
@@ -112,18 +114,20 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
         }
     } else {
         // the shared-memory walk: register-held columns measured slower in this 256-thread kernel
-        block_columns(cs, blockDim.y, Ls, sop, swap != 0, sc, mass[rhs], tid, nthr, false);
+        const SMass<R> sm{mass[rhs], mass[kMaxRhs + rhs]};
+        block_columns(cs, blockDim.y, Ls, sop, swap != 0, sc, sm, tid, nthr, false);
         __syncthreads();
         if (!active) return;
         row_load(mine, res);
     }
-#pragma unroll
-    for (int k = 0; k < 24; ++k) res[k] *= coef;
     if (XPAY) {
         R xv[24];
         xf.load(sr, s, xv);
 #pragma unroll
-        for (int k = 0; k < 24; ++k) res[k] += xv[k];
+        for (int k = 0; k < 24; ++k) res[k] = fma(coef, res[k], xv[k]);
+    } else if (coef != R(1)) {
+#pragma unroll
+        for (int k = 0; k < 24; ++k) res[k] *= coef;
     }
     store_m5(out, out_exp, sr, s, res);
 }
@@ -143,23 +147,20 @@ static int launch_m5_t(mdwf_ctx* c, const M5Launch& m) {
     const R* mass = m.mass ? reinterpret_cast<const R*>(m.mass)
                            : P == MDWF_F64 ? reinterpret_cast<const R*>(c->mass64)
                                            : reinterpret_cast<const R*>(c->mass32);
-    SCoef<R> sc;
-    sc.b5 = (R)c->b5;
-    sc.c5 = (R)c->c5;
-    sc.Mp = (R)(c->b5 * (4.0 - c->M5) + 1.0);
-    sc.Mm = (R)(c->c5 * (4.0 - c->M5) - 1.0);
+    const SCoef<R> sc = make_scoef<R>(c);
+    const R coef = (R)(m.unscaled ? m.coef : m.coef * sop_scale(c, m.sop));
     const double n5 = (double)g.Vh * g.Ls * m.nrhs;
     LaunchScope scope(c, (m.x ? KB_M5_XPAY : KB_M5) * 3 + P, n5 * site_bytes(P) * (m.x ? 3.0 : 2.0),
                       n5 * (144.0 + (m.x ? 24.0 : 0.0)));
     if (m.x) {
         auto k = m5_kernel<P, true>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask,
+        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, coef, g, m.sop, m.swap, sc, m.mask,
                                           m.out_exp);
     } else {
         auto k = m5_kernel<P, false>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, (R)m.coef, g, m.sop, m.swap, sc, m.mask,
+        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, coef, g, m.sop, m.swap, sc, m.mask,
                                           m.out_exp);
     }
     return check_launch();

@@ -443,8 +443,23 @@ __device__ __forceinline__ long long cb_index(const Geom& g, int x, int y, int z
 //   SOP_DENSE: a dense Ls x Ls table (any coefficients)
 enum SOp { SOP_DENSE = 0, SOP_ID = 1, SOP_A = 2, SOP_MPHI = 3, SOP_K = 4, SOP_C = 5, SOP_MEE = 6 };
 
+// The closed-form operators are applied without their constant factor, which the caller folds into a
+// coefficient that it multiplies anyway (sop_scale): with r = M-/M+ and rho = c5/b5
+//   I = M+ (1 + r C),  M_phi = b5 (1 + rho C),  A = (1/M+) A~,  K = (b5/M+) K~,
+//   A~:  Psi_{Ls-1} = q [b_{Ls-1} + kappa sum_{s<Ls-1} (-r)^s b_s],  q = 1 / (1 - kappa (-r)^{Ls-1}),
+//        Psi_s = b_s - r Psi_{s+1}
+//   K~:  (K~ b)_s = Psi_s + rho Psi_{s+1} = b_s + (rho - r) Psi_{s+1},  (K~ b)_{Ls-1} = Psi_{Ls-1} - m rho Psi_0,
+// two and three multiply-adds per real (A: 3.5 operations and a division per column before, K: 5.5). In FP64 this is
+// what the hop epilogues cost: 2 FMAs per clock and SM. With b5 = 0, M_phi and K keep their factor (c5 C, c5 C A).
+// q depends on the mass and is computed on the host ([kMaxRhs] masses, then [kMaxRhs] values of q).
 template <typename R> struct SCoef {
-    R b5, c5, Mp, Mm;
+    R c5, r, rho, krho;  // krho = rho - r
+    R inv;               // 1 / M+ (K with b5 = 0)
+    int b5_zero;
+    R rp[kMaxLs];        // (-r)^s
+};
+template <typename R> struct SMass {
+    R m, q;
 };
 
 // Complex element types for the column tasks (one 8- or 16-byte access each).
@@ -452,24 +467,30 @@ template <typename R> struct CPair;
 template <> struct CPair<float> { typedef float2 T; };
 template <> struct CPair<double> { typedef double2 T; };
 
-// In place on one complex column: element s at base[k(s) * stride] (re, im as
-// one vector), k(s) = up ? s : Ls-1-s. m = this rhs's mass.
+// The weights (w0, w1) of a bidiagonal operator w0 + w1 C.
 template <typename R>
-__device__ __forceinline__ void column_op(R* base, int stride, int Ls, int op, bool up, const SCoef<R>& sc, R m) {
+__device__ __forceinline__ void bidiag_weights(int op, const SCoef<R>& sc, bool& w0, R& w1) {
+    w0 = op == SOP_MEE || (op == SOP_MPHI && !sc.b5_zero);
+    w1 = op == SOP_MEE ? sc.r : op == SOP_MPHI ? (sc.b5_zero ? sc.c5 : sc.rho) : R(1);
+}
+
+// In place on one complex column: element s at base[k(s) * stride] (re, im as
+// one vector), k(s) = up ? s : Ls-1-s.
+template <typename R>
+__device__ __forceinline__ void column_op(R* base, int stride, int Ls, int op, bool up, const SCoef<R>& sc,
+                                          const SMass<R>& sm) {
     typedef typename CPair<R>::T C;
     auto at = [&](int s) -> C* { return reinterpret_cast<C*>(base + (up ? s : Ls - 1 - s) * stride); };
     if (op == SOP_A || op == SOP_K) {
-        const R r = sc.Mm / sc.Mp, kappa = m * r, inv = R(1) / sc.Mp;
-        C last = *at(Ls - 1);
-        R ar = last.x, ai = last.y, pw = kappa;
+        const R r = sc.r, kappa = sm.m * r;
+        R ar = 0, ai = 0;
         for (int s = 0; s < Ls - 1; ++s) {
             const C q = *at(s);
-            ar += pw * q.x;
-            ai += pw * q.y;
-            pw *= -r;
+            ar = fma(sc.rp[s], q.x, ar);
+            ai = fma(sc.rp[s], q.y, ai);
         }
-        const R den = sc.Mp * (R(1) - pw);
-        R pr = ar / den, pi = ai / den;  // Psi_{Ls-1}
+        const C last = *at(Ls - 1);
+        R pr = fma(kappa, ar, last.x) * sm.q, pi = fma(kappa, ai, last.y) * sm.q;  // Psi_{Ls-1}
         const R lr = pr, li = pi;
         if (op == SOP_A) {
             C o; o.x = pr; o.y = pi;
@@ -477,8 +498,8 @@ __device__ __forceinline__ void column_op(R* base, int stride, int Ls, int op, b
             for (int s = Ls - 2; s >= 0; --s) {
                 C* t = at(s);
                 const C b = *t;
-                pr = b.x * inv - r * pr;
-                pi = b.y * inv - r * pi;
+                pr = fma(-r, pr, b.x);
+                pi = fma(-r, pi, b.y);
                 o.x = pr; o.y = pi;
                 *t = o;
             }
@@ -486,69 +507,71 @@ __device__ __forceinline__ void column_op(R* base, int stride, int Ls, int op, b
             for (int s = Ls - 2; s >= 0; --s) {
                 C* t = at(s);
                 const C b = *t;
-                const R nr = b.x * inv - r * pr, ni = b.y * inv - r * pi;  // Psi_s
                 C o;
-                o.x = sc.b5 * nr + sc.c5 * pr;                             // (M_phi Psi)_s
-                o.y = sc.b5 * ni + sc.c5 * pi;
+                if (sc.b5_zero) {
+                    o.x = sc.c5 * (sc.inv * pr);
+                    o.y = sc.c5 * (sc.inv * pi);
+                } else {
+                    o.x = fma(sc.krho, pr, b.x);
+                    o.y = fma(sc.krho, pi, b.y);
+                }
                 *t = o;
-                pr = nr;
-                pi = ni;
+                pr = fma(-r, pr, b.x);
+                pi = fma(-r, pi, b.y);
             }
             C o;  // row Ls-1 wraps to Psi_0 (now in pr, pi) with -m
-            o.x = sc.b5 * lr - m * sc.c5 * pr;
-            o.y = sc.b5 * li - m * sc.c5 * pi;
+            const R w = -sm.m * (sc.b5_zero ? sc.c5 * sc.inv : sc.rho);
+            o.x = fma(w, pr, sc.b5_zero ? R(0) : lr);
+            o.y = fma(w, pi, sc.b5_zero ? R(0) : li);
             *at(Ls - 1) = o;
         }
     } else if (op == SOP_MPHI || op == SOP_C || op == SOP_MEE) {
-        const R w0 = op == SOP_MPHI ? sc.b5 : op == SOP_MEE ? sc.Mp : R(0);
-        const R w1 = op == SOP_MPHI ? sc.c5 : op == SOP_MEE ? sc.Mm : R(1);
+        bool w0;
+        R w1;
+        bidiag_weights(op, sc, w0, w1);
         const C f0 = *at(0);
         C cur = f0;
         for (int s = 0; s < Ls - 1; ++s) {
             const C nxt = *at(s + 1);
             C o;
-            o.x = w0 * cur.x + w1 * nxt.x;
-            o.y = w0 * cur.y + w1 * nxt.y;
+            o.x = fma(w1, nxt.x, w0 ? cur.x : R(0));
+            o.y = fma(w1, nxt.y, w0 ? cur.y : R(0));
             *at(s) = o;
             cur = nxt;
         }
         C o;
-        o.x = w0 * cur.x - m * w1 * f0.x;
-        o.y = w0 * cur.y - m * w1 * f0.y;
+        o.x = fma(-sm.m * w1, f0.x, w0 ? cur.x : R(0));
+        o.y = fma(-sm.m * w1, f0.y, w0 ? cur.y : R(0));
         *at(Ls - 1) = o;
     }
 }
 
-// The closed-form I^-1 (Sec. 3) on a register-held column of LS complex
-// values, element s at v[REV ? LS-1-s : s]: first the last element
-// Psi_{Ls-1} from the whole column, returned in (pr, pi) ...
+// Psi_{Ls-1} of A~ on a register-held column of LS complex values, element s at v[REV ? LS-1-s : s] ...
 template <int LS, bool REV, typename C, typename R>
-__device__ __forceinline__ void a_last(const C* v, R r, R kappa, R Mp, R& pr, R& pi) {
-    R ar = v[REV ? 0 : LS - 1].x, ai = v[REV ? 0 : LS - 1].y, pw = kappa;
+__device__ __forceinline__ void a_last(const C* v, const SCoef<R>& sc, const SMass<R>& sm, R& pr, R& pi) {
+    R ar = v[REV ? LS - 1 : 0].x, ai = v[REV ? LS - 1 : 0].y;
 #pragma unroll
-    for (int s = 0; s < LS - 1; ++s) {
-        ar += pw * v[REV ? LS - 1 - s : s].x;
-        ai += pw * v[REV ? LS - 1 - s : s].y;
-        pw *= -r;
+    for (int s = 1; s < LS - 1; ++s) {
+        ar = fma(sc.rp[s], v[REV ? LS - 1 - s : s].x, ar);
+        ai = fma(sc.rp[s], v[REV ? LS - 1 - s : s].y, ai);
     }
-    const R den = Mp * (R(1) - pw);
-    pr = ar / den;
-    pi = ai / den;
+    const R kappa = sm.m * sc.r;
+    pr = fma(kappa, ar, v[REV ? 0 : LS - 1].x) * sm.q;
+    pi = fma(kappa, ai, v[REV ? 0 : LS - 1].y) * sm.q;
 }
 
-// ... then, with Psi_{Ls-1} in place, Psi_s = v_s / M+ - (M- / M+) Psi_{s+1}
-// from s = Ls-2 down, in place: v becomes I^-1 v.
+// ... then, with Psi_{Ls-1} in place, Psi_s = v_s - r Psi_{s+1} from s = Ls-2 down: v becomes A~ v.
 template <int LS, bool REV, typename C, typename R>
-__device__ __forceinline__ void a_solve(C* v, R r, R kappa, R inv, R Mp) {
+__device__ __forceinline__ void a_solve(C* v, const SCoef<R>& sc, const SMass<R>& sm) {
     R pr, pi;
-    a_last<LS, REV>(v, r, kappa, Mp, pr, pi);
+    a_last<LS, REV>(v, sc, sm, pr, pi);
     v[REV ? 0 : LS - 1].x = pr;
     v[REV ? 0 : LS - 1].y = pi;
 #pragma unroll
     for (int s = LS - 2; s >= 0; --s) {
         C& e = v[REV ? LS - 1 - s : s];
-        pr = e.x * inv - r * pr;
-        pi = e.y * inv - r * pi;
+        pr = fma(-sc.r, pr, e.x);
+        pi = fma(-sc.r, pi, e.y);
         e.x = pr;
         e.y = pi;
     }
@@ -556,43 +579,45 @@ __device__ __forceinline__ void a_solve(C* v, R r, R kappa, R inv, R Mp) {
 
 // column_op with the column held in registers (Ls known at compile time): all
 // Ls elements are loaded at once, the recursion runs on registers, and all are
-// stored back; the arithmetic is that of column_op.
+// stored back; the arithmetic is that of column_op. (C, and with b5 = 0 M_phi and K,
+// which no tuned path uses, go through column_op.)
 template <int LS, typename R>
-__device__ __forceinline__ void column_op_reg(R* base, int stride, int op, bool up, const SCoef<R>& sc, R m) {
+__device__ __forceinline__ void column_op_reg(R* base, int stride, int op, bool up, const SCoef<R>& sc,
+                                              const SMass<R>& sm) {
     typedef typename CPair<R>::T C;
+    if (op == SOP_C || (sc.b5_zero && (op == SOP_K || op == SOP_MPHI))) {
+        column_op(base, stride, LS, op, up, sc, sm);
+        return;
+    }
     C v[LS];
 #pragma unroll
     for (int s = 0; s < LS; ++s) v[s] = *reinterpret_cast<const C*>(base + (up ? s : LS - 1 - s) * stride);
-    if (op == SOP_A || op == SOP_K) {
-        const R r = sc.Mm / sc.Mp, kappa = m * r, inv = R(1) / sc.Mp;
-        if (op == SOP_A) {
-            a_solve<LS, false>(v, r, kappa, inv, sc.Mp);
-        } else {
-            R pr, pi;
-            a_last<LS, false>(v, r, kappa, sc.Mp, pr, pi);  // Psi_{Ls-1}
-            const R lr = pr, li = pi;
+    if (op == SOP_A) {
+        a_solve<LS, false>(v, sc, sm);
+    } else if (op == SOP_K) {
+        R pr, pi;
+        a_last<LS, false>(v, sc, sm, pr, pi);  // Psi_{Ls-1}
+        const R lr = pr, li = pi;
 #pragma unroll
-            for (int s = LS - 2; s >= 0; --s) {
-                const R nr = v[s].x * inv - r * pr, ni = v[s].y * inv - r * pi;  // Psi_s
-                v[s].x = sc.b5 * nr + sc.c5 * pr;                               // (M_phi Psi)_s
-                v[s].y = sc.b5 * ni + sc.c5 * pi;
-                pr = nr;
-                pi = ni;
-            }
-            v[LS - 1].x = sc.b5 * lr - m * sc.c5 * pr;
-            v[LS - 1].y = sc.b5 * li - m * sc.c5 * pi;
+        for (int s = LS - 2; s >= 0; --s) {
+            const C b = v[s];
+            v[s].x = fma(sc.krho, pr, b.x);
+            v[s].y = fma(sc.krho, pi, b.y);
+            pr = fma(-sc.r, pr, b.x);
+            pi = fma(-sc.r, pi, b.y);
         }
-    } else if (op == SOP_MPHI || op == SOP_C || op == SOP_MEE) {
-        const R w0 = op == SOP_MPHI ? sc.b5 : op == SOP_MEE ? sc.Mp : R(0);
-        const R w1 = op == SOP_MPHI ? sc.c5 : op == SOP_MEE ? sc.Mm : R(1);
+        v[LS - 1].x = fma(-sm.m * sc.rho, pr, lr);
+        v[LS - 1].y = fma(-sm.m * sc.rho, pi, li);
+    } else if (op == SOP_MPHI || op == SOP_MEE) {
+        const R w1 = op == SOP_MPHI ? sc.rho : sc.r;
         const C f0 = v[0];
 #pragma unroll
         for (int s = 0; s < LS - 1; ++s) {
-            v[s].x = w0 * v[s].x + w1 * v[s + 1].x;
-            v[s].y = w0 * v[s].y + w1 * v[s + 1].y;
+            v[s].x = fma(w1, v[s + 1].x, v[s].x);
+            v[s].y = fma(w1, v[s + 1].y, v[s].y);
         }
-        v[LS - 1].x = w0 * v[LS - 1].x - m * w1 * f0.x;
-        v[LS - 1].y = w0 * v[LS - 1].y - m * w1 * f0.y;
+        v[LS - 1].x = fma(-sm.m * w1, f0.x, v[LS - 1].x);
+        v[LS - 1].y = fma(-sm.m * w1, f0.y, v[LS - 1].y);
     } else {
         return;
     }
@@ -601,12 +626,13 @@ __device__ __forceinline__ void column_op_reg(R* base, int stride, int op, bool 
 }
 
 template <typename R>
-__device__ __forceinline__ void column_op_any(R* base, int stride, int Ls, int op, bool up, const SCoef<R>& sc, R m) {
+__device__ __forceinline__ void column_op_any(R* base, int stride, int Ls, int op, bool up, const SCoef<R>& sc,
+                                              const SMass<R>& sm) {
     switch (Ls) {
-        case 8: column_op_reg<8>(base, stride, op, up, sc, m); return;
-        case 12: column_op_reg<12>(base, stride, op, up, sc, m); return;
-        case 16: column_op_reg<16>(base, stride, op, up, sc, m); return;
-        default: column_op(base, stride, Ls, op, up, sc, m); return;
+        case 8: column_op_reg<8>(base, stride, op, up, sc, sm); return;
+        case 12: column_op_reg<12>(base, stride, op, up, sc, sm); return;
+        case 16: column_op_reg<16>(base, stride, op, up, sc, sm); return;
+        default: column_op(base, stride, Ls, op, up, sc, sm); return;
     }
 }
 
@@ -658,7 +684,7 @@ __host__ __device__ inline int site_stride(int Ls) {
 // through shared memory.
 template <int LSR = -1, typename R>
 __device__ __forceinline__ void block_columns(R* hs, int SB, int Ls, int op, bool swap, const SCoef<R>& sc,
-                                              R m, int tid, int nthr, bool in_registers = true) {
+                                              const SMass<R>& sm, int tid, int nthr, bool in_registers = true) {
     const int ss = site_stride(Ls);
     const int per = SB * 6, half = (per + 31) / 32 * 32;
     for (int t = tid; t < 2 * half; t += nthr) {
@@ -666,39 +692,39 @@ __device__ __forceinline__ void block_columns(R* hs, int SB, int Ls, int op, boo
         if (r >= per) continue;
         const int ly = r / 6, j = chir * 6 + (r - 6 * (r / 6));
         const bool up = (chir == 1) != swap;  // P- uses N' unless the adjoint swaps
-        if constexpr (LSR > 0) column_op_reg<LSR>(hs + (size_t)ly * ss + 2 * j, kRowStride, op, up, sc, m);
-        else if (in_registers) column_op_any(hs + (size_t)ly * ss + 2 * j, kRowStride, Ls, op, up, sc, m);
-        else column_op(hs + (size_t)ly * ss + 2 * j, kRowStride, Ls, op, up, sc, m);
+        if constexpr (LSR > 0) column_op_reg<LSR>(hs + (size_t)ly * ss + 2 * j, kRowStride, op, up, sc, sm);
+        else if (in_registers) column_op_any(hs + (size_t)ly * ss + 2 * j, kRowStride, Ls, op, up, sc, sm);
+        else column_op(hs + (size_t)ly * ss + 2 * j, kRowStride, Ls, op, up, sc, sm);
     }
 }
 
 // The column pass of the fused t, v epilogue (closed form, Ls = LS): with y
-// staged in the rows, each column becomes t = A y, its share of |t|^2 goes
-// to the returned sum, and then v = A^dag t, which for one chirality is the
-// same recursion run from the other end of the column; v replaces y in the
+// staged in the rows, each column becomes t = A~ y, its share of |t|^2 goes
+// to the returned sum, and then A~^dag t, which for one chirality is the
+// same recursion run from the other end of the column, replaces y in the
 // rows. Tasks as in block_columns.
 template <int LS, typename R>
-__device__ __forceinline__ R column_a_adag_reg(R* base, int stride, bool up, const SCoef<R>& sc, R m) {
+__device__ __forceinline__ R column_a_adag_reg(R* base, int stride, bool up, const SCoef<R>& sc, const SMass<R>& sm) {
     typedef typename CPair<R>::T C;
     C v[LS];
 #pragma unroll
     for (int s = 0; s < LS; ++s) v[s] = *reinterpret_cast<const C*>(base + (up ? s : LS - 1 - s) * stride);
-    const R r = sc.Mm / sc.Mp, kappa = m * r, inv = R(1) / sc.Mp;
-    a_solve<LS, false>(v, r, kappa, inv, sc.Mp);
+    a_solve<LS, false>(v, sc, sm);
     R sq = 0;
 #pragma unroll
     for (int s = 0; s < LS; ++s) {
         sq = fma(v[s].x, v[s].x, sq);
         sq = fma(v[s].y, v[s].y, sq);
     }
-    a_solve<LS, true>(v, r, kappa, inv, sc.Mp);
+    a_solve<LS, true>(v, sc, sm);
 #pragma unroll
     for (int s = 0; s < LS; ++s) *reinterpret_cast<C*>(base + (up ? s : LS - 1 - s) * stride) = v[s];
     return sq;
 }
 
 template <int LS, typename R>
-__device__ __forceinline__ R block_columns_a_adag(R* hs, int SB, const SCoef<R>& sc, R m, int tid, int nthr) {
+__device__ __forceinline__ R block_columns_a_adag(R* hs, int SB, const SCoef<R>& sc, const SMass<R>& sm, int tid,
+                                                  int nthr) {
     const int ss = site_stride(LS);
     const int per = SB * 6, half = (per + 31) / 32 * 32;
     R sq = 0;
@@ -706,7 +732,7 @@ __device__ __forceinline__ R block_columns_a_adag(R* hs, int SB, const SCoef<R>&
         const int chir = t >= half ? 1 : 0, r = t - chir * half;
         if (r >= per) continue;
         const int ly = r / 6, j = chir * 6 + (r - 6 * (r / 6));
-        sq += column_a_adag_reg<LS>(hs + (size_t)ly * ss + 2 * j, kRowStride, chir == 1, sc, m);
+        sq += column_a_adag_reg<LS>(hs + (size_t)ly * ss + 2 * j, kRowStride, chir == 1, sc, sm);
     }
     return sq;
 }
@@ -875,19 +901,58 @@ template <class L> inline void set_sop(const mdwf_ctx* c, int prec, int sop, int
     }
 }
 
+// The constant factor that a launch of s-operator sop leaves out (SCoef); 1 for dense tables.
+inline double sop_scale(const mdwf_ctx* c, int sop) {
+    if (sop == SOP_DENSE) return 1.0;
+    const double Mp = c->b5 * (4.0 - c->M5) + 1.0;
+    const bool z = c->b5 == 0.0;
+    switch (sop) {
+        case SOP_A: return 1.0 / Mp;
+        case SOP_MEE: return Mp;
+        case SOP_MPHI: return z ? 1.0 : c->b5;
+        case SOP_K: return z ? 1.0 : c->b5 / Mp;
+    }
+    return 1.0;
+}
+// the factor of s-operator sop as this context applies it
+inline double ctx_scale(const mdwf_ctx* c, int sop) { return c->dense_s ? 1.0 : sop_scale(c, sop); }
+
+template <typename R> inline SCoef<R> make_scoef(const mdwf_ctx* c) {
+    SCoef<R> sc;
+    const double Mp = c->b5 * (4.0 - c->M5) + 1.0, Mm = c->c5 * (4.0 - c->M5) - 1.0;
+    const double r = Mp != 0.0 ? Mm / Mp : 0.0, rho = c->b5 != 0.0 ? c->c5 / c->b5 : 0.0;
+    sc.c5 = (R)c->c5;
+    sc.r = (R)r;
+    sc.rho = (R)rho;
+    sc.krho = (R)(rho - r);
+    sc.inv = (R)(Mp != 0.0 ? 1.0 / Mp : 0.0);
+    sc.b5_zero = c->b5 == 0.0;
+    double pw = 1.0;
+    for (int s = 0; s < kMaxLs; ++s, pw *= -r) sc.rp[s] = (R)pw;
+    return sc;
+}
+// q of SCoef for mass m
+inline double scoef_q(const mdwf_ctx* c, double m) {
+    const double Mp = c->b5 * (4.0 - c->M5) + 1.0, r = Mp != 0.0 ? (c->c5 * (4.0 - c->M5) - 1.0) / Mp : 0.0;
+    double pw = m * r;
+    for (int s = 0; s < c->g.Ls - 1; ++s) pw *= -r;
+    return 1.0 / (1.0 - pw);
+}
+
 // launchers (dslash.cu, m5.cu)
 struct HopLaunch {
     void* out;
     const void* in;
     const void* x;        // xpay addend (same parity as out) or nullptr
     double coef;          // result = coef * Mat (H in) [+ x]
+    int unscaled;         // 1: Mat without its constant factor (sop_scale), which the caller accounts for
     int out_parity;
     int dagger;           // 1: hopping term of D_W^dag (projector signs flipped)
     const void* mat;      // dense table of the output Ls x Ls matrix (sop == SOP_DENSE), per rhs
     const void* mat2;     // dense table of A^dag for the FUSE_T epilogue (sop == SOP_DENSE)
     int sop;              // output s-operator (SOp)
     int swap;             // 1: the adjoint (chirality-swapped) s-operator
-    const void* mass;     // per-rhs masses (double for F64, float otherwise)
+    const void* mass;     // per-rhs masses and, kMaxRhs further, their q (SCoef); double for F64, else float
     int nrhs;
     // FP64 hops outside t-slabs read a fixed-point field (fx.cuh): its exponents (required), and, where the
     // output (out, or out2 of fuse = 1) is to be fixed-point too, its exponents
@@ -920,6 +985,7 @@ struct M5Launch {
     const void* in;
     const void* x;    // optional addend
     double coef;      // out = coef * Mat in [+ x]
+    int unscaled;     // 1: Mat without its constant factor (sop_scale)
     const void* mat;  // dense table (sop == SOP_DENSE)
     int sop;
     int swap;

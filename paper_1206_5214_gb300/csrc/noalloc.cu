@@ -32,8 +32,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[2 * kNoAllocFie
 // exponents of the two fields where they are fixed-point (the FP64 operator: 192 bytes a 5d site)
 constexpr size_t kNoAllocExps = kNoAllocFieldBytes / 192;
 static __device__ __align__(256) int g_noalloc_exp[2 * kNoAllocExps];
-static __device__ __align__(256) double g_noalloc_mass64[64];
-static __device__ __align__(256) float g_noalloc_mass32[64];
+static __device__ __align__(256) double g_noalloc_mass64[2 * kMaxRhs];  // masses, then their q (SCoef)
+static __device__ __align__(256) float g_noalloc_mass32[2 * kMaxRhs];
 
 struct NoAllocAddrs {
     bool ready = false;
@@ -70,8 +70,7 @@ static int noalloc_setup(int device, NoAllocAddrs** out) {
 
 // The masses of one call, passed by value.
 struct NoAllocMasses {
-    double m64[64];
-    float m32[64];
+    double m64[kMaxRhs], q64[kMaxRhs];
     int n;
 };
 
@@ -79,7 +78,9 @@ __global__ void k_noalloc_masses(NoAllocMasses m) {
     const int r = threadIdx.x;
     if (r < m.n) {
         g_noalloc_mass64[r] = m.m64[r];
-        g_noalloc_mass32[r] = m.m32[r];
+        g_noalloc_mass64[kMaxRhs + r] = m.q64[r];
+        g_noalloc_mass32[r] = (float)m.m64[r];
+        g_noalloc_mass32[kMaxRhs + r] = (float)m.q64[r];
     }
 }
 
@@ -138,7 +139,7 @@ extern "C" int mdwf_apply_noalloc(mdwf_ctx* c, void* out, const void* in, int pr
     ms.n = nrhs;
     for (int r = 0; r < nrhs; ++r) {
         ms.m64[r] = mf_per_rhs ? mf_per_rhs[r] : c->mf;
-        ms.m32[r] = (float)ms.m64[r];
+        ms.q64[r] = scoef_q(c, ms.m64[r]);
     }
     k_noalloc_masses<<<1, 64, 0, c->stream>>>(ms);
     if ((st = check_launch())) return st;
