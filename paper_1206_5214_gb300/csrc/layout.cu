@@ -5,68 +5,81 @@
 
 namespace mdwf {
 
-template <int P>
-__global__ void import_odd_kernel(Field<P> dst, const double* __restrict__ src, Geom g, int nrhs) {
-    typedef typename PrecTraits<P>::real R;
-    const long long n = (long long)nrhs * g.Vh * g.Ls;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(i % g.Ls);
-        const long long sr = i / g.Ls;  // rhs * Vh + site
-        const long long rhs = sr / g.Vh, site = sr % g.Vh;
-        const double* p = src + ((rhs * g.Ls + s) * g.Vh + site) * 24;
-        R v[24];
-#pragma unroll
-        for (int k = 0; k < 24; ++k) v[k] = (R)p[k];
-        dst.store(sr, s, v);
-    }
-}
+// User fields <-> internal fields. FULL: the user field is [rhs][s][2 Vh sites][24] and its sites alternate between
+// the two parities (internal site = lexicographic index / 2); else it is [rhs][s][Vh odd sites][24] (odd only).
+// A block takes SB consecutive user sites and their Ls slices: for each slice the user field holds SB 192 contiguous
+// bytes, read (or written) with consecutive 16-byte accesses, and the internal field is accessed by its own chunks;
+// shared memory turns one into the other. (One thread per (site, s) that walks its 192 bytes in the user field,
+// with the slices of a site far apart, moved 1.8 TB/s: import and export of 16^3 x 32 x 16 FP32 took 341 us, now
+// 133 us, 4.5 TB/s.)
+// Rows of 13 double2 put the 16-byte row accesses of 8 consecutive threads on distinct banks.
+constexpr int kLayoutRow = 13;
 
-template <int P>
-__global__ void export_odd_kernel(double* __restrict__ dst, Field<P> src, Geom g, int nrhs) {
+template <int P, bool FULL, bool TO_INTERNAL>
+__global__ void __launch_bounds__(128) layout_kernel(Field<P> even, Field<P> odd, double* user, Geom g, int nrhs) {
     typedef typename PrecTraits<P>::real R;
-    const long long n = (long long)nrhs * g.Vh * g.Ls;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(i % g.Ls);
-        const long long sr = i / g.Ls;
-        const long long rhs = sr / g.Vh, site = sr % g.Vh;
-        R v[24];
-        src.load(sr, s, v);
-        double* p = dst + ((rhs * g.Ls + s) * g.Vh + site) * 24;
-#pragma unroll
-        for (int k = 0; k < 24; ++k) p[k] = (double)v[k];
-    }
-}
-
-// full user field [rhs][s][V][24] <-> internal even / odd fields
-template <int P, bool TO_INTERNAL>
-__global__ void full_kernel(Field<P> even, Field<P> odd, double* full, Geom g, int nrhs) {
-    typedef typename PrecTraits<P>::real R;
-    const long long V = 2 * g.Vh;
-    const long long n = (long long)nrhs * V * g.Ls;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(i % g.Ls);
-        const long long r = i / g.Ls;
-        const long long rhs = r / V, lex = r % V;
-        long long q = lex;
+    extern __shared__ __align__(16) double2 tile[];  // [site of the block][s][kLayoutRow]
+    const int Ls = g.Ls, SB = blockDim.y, s = threadIdx.x, ly = threadIdx.y;
+    const int tid = ly * Ls + s, nthr = Ls * SB;
+    const long long N = FULL ? 2 * g.Vh : g.Vh;
+    const long long per = (N + SB - 1) / SB;
+    const long long rhs = blockIdx.x / per, base = (blockIdx.x % per) * SB;
+    const int live = (int)(N - base < SB ? N - base : SB);  // sites of this block
+    const long long site = base + ly;
+    int par = 1;
+    long long sr = rhs * g.Vh + site;
+    if (FULL) {
+        long long q = site;
         const int x = (int)(q % g.X); q /= g.X;
         const int y = (int)(q % g.Y); q /= g.Y;
         const int z = (int)(q % g.Z); q /= g.Z;
-        const int t = (int)q;
-        const int par = (x + y + z + t) & 1;
-        const long long sr = rhs * g.Vh + (lex >> 1);
-        double* p = full + ((rhs * g.Ls + s) * V + lex) * 24;
+        par = (x + y + z + (int)q) & 1;
+        sr = rhs * g.Vh + (site >> 1);
+    }
+    double2* row = tile + (size_t)tid * kLayoutRow;
+    // a caller's doubles need not be 16-byte aligned (so `user` must not be a double2*: the compiler may then
+    // join the two 8-byte accesses)
+    const bool wide = (reinterpret_cast<size_t>(user) & 15) == 0;
+    // (slice, site of the block, 16-byte word) of the user side, words fastest
+    auto copy_user = [&](auto f) {
+        for (int i = tid; i < Ls * live * 12; i += nthr) {
+            const int w = i % 12, r = i / 12, l = r % live, t = r / live;
+            f(user + (((rhs * Ls + t) * N + base + l) * 12 + w) * 2, tile + ((size_t)l * Ls + t) * kLayoutRow + w);
+        }
+    };
+    if (TO_INTERNAL) {
+        copy_user([=](const double* u, double2* t) {
+            if (wide) *t = __ldg(reinterpret_cast<const double2*>(u));
+            else *t = make_double2(__ldg(u), __ldg(u + 1));
+        });
+        __syncthreads();
+        if (ly >= live) return;
         R v[24];
-        if (TO_INTERNAL) {
 #pragma unroll
-            for (int k = 0; k < 24; ++k) v[k] = (R)p[k];
-            if (par) odd.store(sr, s, v);
-            else even.store(sr, s, v);
-        } else {
+        for (int k = 0; k < 12; ++k) {
+            const double2 d = row[k];
+            v[2 * k] = (R)d.x;
+            v[2 * k + 1] = (R)d.y;
+        }
+        if (par) odd.store(sr, s, v);
+        else even.store(sr, s, v);
+    } else {
+        if (ly < live) {
+            R v[24];
             if (par) odd.load(sr, s, v);
             else even.load(sr, s, v);
 #pragma unroll
-            for (int k = 0; k < 24; ++k) p[k] = (double)v[k];
+            for (int k = 0; k < 12; ++k) row[k] = make_double2((double)v[2 * k], (double)v[2 * k + 1]);
         }
+        __syncthreads();
+        copy_user([=](double* u, const double2* t) {
+            if (wide) {
+                *reinterpret_cast<double2*>(u) = *t;
+            } else {
+                u[0] = t->x;
+                u[1] = t->y;
+            }
+        });
     }
 }
 
@@ -151,56 +164,43 @@ static dim3 grid_for(long long n, int threads) {
     return dim3((unsigned)b);
 }
 
-template <int P>
-static int import_t(mdwf_ctx* c, void* dst, const double* src, int nrhs) {
-    const long long n = (long long)nrhs * c->g.Vh * c->g.Ls;
-    LaunchScope scope(c, KB_LAYOUT * 3 + P, n * (192.0 + site_bytes(P)), 0.0);
-    import_odd_kernel<P><<<grid_for(n, 256), 256, 0, c->stream>>>(make_field<P>(dst, c->g, nrhs), src, c->g, nrhs);
-    return check_launch();
-}
-
-template <int P>
-static int export_t(mdwf_ctx* c, double* dst, const void* src, int nrhs) {
-    const long long n = (long long)nrhs * c->g.Vh * c->g.Ls;
-    LaunchScope scope(c, KB_LAYOUT * 3 + P, n * (192.0 + site_bytes(P)), 0.0);
-    export_odd_kernel<P><<<grid_for(n, 256), 256, 0, c->stream>>>(dst, make_field<P>(const_cast<void*>(src), c->g, nrhs),
-                                                                   c->g, nrhs);
-    return check_launch();
-}
-
-template <int P, bool TO>
-static int full_t(mdwf_ctx* c, void* even, void* odd, double* full, int nrhs) {
-    const long long n = (long long)nrhs * 2 * c->g.Vh * c->g.Ls;
-    LaunchScope scope(c, KB_LAYOUT * 3 + P, n * (192.0 + site_bytes(P)), 0.0);
-    full_kernel<P, TO><<<grid_for(n, 256), 256, 0, c->stream>>>(make_field<P>(even, c->g, nrhs),
-                                                                  make_field<P>(odd, c->g, nrhs), full, c->g, nrhs);
+template <int P, bool FULL, bool TO>
+static int layout_t(mdwf_ctx* c, void* even, void* odd, const double* user, int nrhs) {
+    const Geom& g = c->g;
+    const long long N = FULL ? 2 * g.Vh : g.Vh;
+    const int SB = 128 / g.Ls;
+    LaunchScope scope(c, KB_LAYOUT * 3 + P, (double)nrhs * N * g.Ls * (192.0 + site_bytes(P)), 0.0);
+    layout_kernel<P, FULL, TO><<<dim3((unsigned)((N + SB - 1) / SB * nrhs)), dim3(g.Ls, SB),
+                                 sizeof(double2) * kLayoutRow * g.Ls * SB, c->stream>>>(
+        make_field<P>(even, g, nrhs), make_field<P>(odd, g, nrhs),
+        const_cast<double*>(user), g, nrhs);
     return check_launch();
 }
 
 int launch_import_odd(mdwf_ctx* c, void* dst, const double* src, int prec, int nrhs) {
     switch (prec) {
-        case MDWF_F64: return import_t<MDWF_F64>(c, dst, src, nrhs);
-        case MDWF_F32: return import_t<MDWF_F32>(c, dst, src, nrhs);
-        case MDWF_F16N: return import_t<MDWF_F16N>(c, dst, src, nrhs);
+        case MDWF_F64: return layout_t<MDWF_F64, false, true>(c, dst, dst, src, nrhs);
+        case MDWF_F32: return layout_t<MDWF_F32, false, true>(c, dst, dst, src, nrhs);
+        case MDWF_F16N: return layout_t<MDWF_F16N, false, true>(c, dst, dst, src, nrhs);
     }
     return MDWF_EINVAL;
 }
 
 int launch_export_odd(mdwf_ctx* c, double* dst, const void* src, int prec, int nrhs) {
+    void* f = const_cast<void*>(src);
     switch (prec) {
-        case MDWF_F64: return export_t<MDWF_F64>(c, dst, src, nrhs);
-        case MDWF_F32: return export_t<MDWF_F32>(c, dst, src, nrhs);
-        case MDWF_F16N: return export_t<MDWF_F16N>(c, dst, src, nrhs);
+        case MDWF_F64: return layout_t<MDWF_F64, false, false>(c, f, f, dst, nrhs);
+        case MDWF_F32: return layout_t<MDWF_F32, false, false>(c, f, f, dst, nrhs);
+        case MDWF_F16N: return layout_t<MDWF_F16N, false, false>(c, f, f, dst, nrhs);
     }
     return MDWF_EINVAL;
 }
 
 int launch_split_full(mdwf_ctx* c, void* dst_even, void* dst_odd, const double* full, int prec, int nrhs) {
-    double* f = const_cast<double*>(full);
     switch (prec) {
-        case MDWF_F64: return full_t<MDWF_F64, true>(c, dst_even, dst_odd, f, nrhs);
-        case MDWF_F32: return full_t<MDWF_F32, true>(c, dst_even, dst_odd, f, nrhs);
-        case MDWF_F16N: return full_t<MDWF_F16N, true>(c, dst_even, dst_odd, f, nrhs);
+        case MDWF_F64: return layout_t<MDWF_F64, true, true>(c, dst_even, dst_odd, full, nrhs);
+        case MDWF_F32: return layout_t<MDWF_F32, true, true>(c, dst_even, dst_odd, full, nrhs);
+        case MDWF_F16N: return layout_t<MDWF_F16N, true, true>(c, dst_even, dst_odd, full, nrhs);
     }
     return MDWF_EINVAL;
 }
@@ -209,9 +209,9 @@ int launch_join_full(mdwf_ctx* c, double* full, const void* even, const void* od
     void* e = const_cast<void*>(even);
     void* o = const_cast<void*>(odd);
     switch (prec) {
-        case MDWF_F64: return full_t<MDWF_F64, false>(c, e, o, full, nrhs);
-        case MDWF_F32: return full_t<MDWF_F32, false>(c, e, o, full, nrhs);
-        case MDWF_F16N: return full_t<MDWF_F16N, false>(c, e, o, full, nrhs);
+        case MDWF_F64: return layout_t<MDWF_F64, true, false>(c, e, o, full, nrhs);
+        case MDWF_F32: return layout_t<MDWF_F32, true, false>(c, e, o, full, nrhs);
+        case MDWF_F16N: return layout_t<MDWF_F16N, true, false>(c, e, o, full, nrhs);
     }
     return MDWF_EINVAL;
 }
