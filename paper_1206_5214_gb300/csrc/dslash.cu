@@ -18,6 +18,25 @@ int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs) {
     return sb < 1 ? 1 : sb;
 }
 
+// The block shape of a hop launch. Where the whole s-columns of 128 threads make so few blocks that the time of a
+// hop is that of one thread's chain of eight neighbours, four threads share a column (STAGE 5 of the kernel). M alone,
+// ordinary and split form, by the number of ordinary blocks:
+//   FP32: 8 blocks 16.4 and 13.7 us, 128 blocks 17.0 and 14.4, 140 blocks 20.5 and 16.5, 256 blocks 16.5 and 20.5;
+//   FP64: 8 blocks 49 and 30 us, 32 blocks 51 and 33, 128 blocks 51 and 56, 256 blocks 65 and 96.
+// FP32 gains while the ordinary form leaves an SM at most one block; FP64, whose blocks wait for the integer
+// and FP64 pipes more than for memory, only while the four times as many split blocks still have an SM each.
+// Not for FP16+norm (its sums would round differently), a tuned block shape or a chosen load strategy.
+constexpr int kSplitBlocksF32 = 152, kSplitBlocksF64 = 152 / 4;
+HopShape hop_shape(const mdwf_ctx* c, int prec, int nrhs) {
+    const int sb = hop_sites_per_block(c, prec, nrhs);
+    const long long blocks = (c->g.Vh + sb - 1) / sb * nrhs;
+    const bool tuned = nrhs >= 1 && nrhs <= 64 && c->sb_tune[prec][nrhs] > 0;
+    if (prec == MDWF_F16N || c->slab || tuned || c->hop_stage[prec] != 0 || 
+        blocks > (prec == MDWF_F64 ? kSplitBlocksF64 : kSplitBlocksF32))
+        return {sb, false};
+    return {32 / c->g.Ls, true};
+}
+
 // The fused iteration drops its t field when the FUSE_R epilogue can rebuild
 // t = I^dag v by shuffles: FP32 or FP16+norm operators at Ls = 16 with the
 // closed-form s-operators, whole s-columns in every warp (an even number of
@@ -25,13 +44,13 @@ int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs) {
 // time (not the two shared-memory staging modes).
 bool hop_no_t_ok(const mdwf_ctx* c, int prec, int nrhs) {
     if (prec == MDWF_F64 || c->g.Ls != 16 || c->dense_s || c->sdep) return false;
-    if (hop_sites_per_block(c, prec, nrhs) & 1) return false;
+    if (hop_shape(c, prec, nrhs).sites & 1) return false;
     const int mode = c->hop_stage[prec];
     return mode != 1 && mode != 2;
 }
 
 int hop_blocks(const mdwf_ctx* c, int prec, int nrhs) {
-    const int SB = hop_sites_per_block(c, prec, nrhs);
+    const int SB = hop_shape(c, prec, nrhs).sites;
     return (int)((c->g.Vh + SB - 1) / SB);
 }
 

@@ -95,11 +95,12 @@ struct FxHop {
     int xf, xb;            // their exponents
 };
 
-// The eight terms of one (site, s): acc = H w as doubles. False where a neighbour or a link is not
+// Terms t0, t0 + DT, ... of the eight of one (site, s), t = 0..3 the forward ones, 4..7 the backward ones: their sum
+// as integers at the exponent `top` of the largest term of all eight. False where a neighbour or a link is not
 // finite (the caller then takes the FP64 arithmetic).
-template <bool DAG>
-__device__ __forceinline__ bool fx_hop(double* out, const FxHop& fx, const Geom& g, int out_parity, const int* nbi,
-                                       long long site, int s, long long rbase) {
+template <bool DAG, int DT>
+__device__ __forceinline__ bool fx_terms(long long* acc, int& top, int t0, const FxHop& fx, const Geom& g,
+                                         int out_parity, const int* nbi, long long site, int s, long long rbase) {
     constexpr int SF = DAG ? +1 : -1;
     // the exponent of term t, t = 0..3 the forward terms, 4..7 the backward ones
     auto term_exponent = [&](int t, long long j, long long l) {
@@ -110,20 +111,17 @@ __device__ __forceinline__ bool fx_hop(double* out, const FxHop& fx, const Geom&
     auto link_of = [&](int t, long long j) {
         return ((long long)(t < 4 ? out_parity : 1 - out_parity) * 4 + (t & 3)) * g.Vh + (t < 4 ? site : j);
     };
-    int top = kFxZero * 4;
+    top = kFxZero * 4;
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const long long j = __ldg(nbi + t);
         top = max(top, term_exponent(t, j, link_of(t, j)));
     }
     if (top >= kFxRawMin) return false;
-    long long acc[24];
-#pragma unroll
-    for (int k = 0; k < 24; ++k) acc[k] = 0;
     // One body for the eight terms (the spin parts by uniform branches): unrolled, the compiler moves the loads of
     // later terms up and spills.
 #pragma unroll 1
-    for (int t = 0; t < 8; ++t) {
+    for (int t = t0; t < 8; t += DT) {
         const long long j = __ldg(nbi + t), l = link_of(t, j);
         const int sh = min(top - term_exponent(t, j, l), 63);
         long long h[12], gg[12];
@@ -161,6 +159,11 @@ __device__ __forceinline__ bool fx_hop(double* out, const FxHop& fx, const Geom&
             default: fx_reconstruct<3, -SF, true>(acc, gg);
         }
     }
+    return true;
+}
+
+// The sum of the eight terms as doubles.
+__device__ __forceinline__ void fx_finish(double* out, const long long* acc, int top) {
     // one unit of acc is 2^64 2^(e - kFxFieldBias) 2^(e' - kFxLinkBias), e + e' = top
     const int x = top - kFxFieldBias - kFxLinkBias + 64;
     if (fx_scale_safe(x)) {
@@ -172,7 +175,6 @@ __device__ __forceinline__ bool fx_hop(double* out, const FxHop& fx, const Geom&
 #pragma unroll
         for (int k = 0; k < 24; ++k) out[k] = fx_to_double(acc[k], 0) * f1 * f2;
     }
-    return true;
 }
 
 }  // namespace mdwf

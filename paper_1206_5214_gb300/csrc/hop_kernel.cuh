@@ -183,7 +183,9 @@ __device__ __forceinline__ void hop_pair64(double* acc, const IN& in, const Gaug
 // read just before its term so that none is held in a register across terms
 template <int P, int MU, bool DAG, bool DD = false, typename IN, typename R>
 __device__ __forceinline__ void hop_dir(R* acc, const IN& in, const Gauge<P>& U, const HopParams<R>& hp,
-                                        const int* nbi, long long site, int s, long long rbase, int rhs = 0) {
+                                        const int* nbi, long long site, int s, long long rbase, int rhs = 0,
+                                        R* accb = nullptr) {
+    // accb: where the backward term goes if not to acc (FP32 / FP16, the split form)
     if constexpr (P == MDWF_F64) {
         if (!(MU == 3 && (hp.chem || DD))) {
             hop_pair64<MU, DAG>(acc, in, U, hp, nbi, site, s, rbase);
@@ -242,7 +244,7 @@ __device__ __forceinline__ void hop_dir(R* acc, const IN& in, const Gauge<P>& U,
         project<MU, -SF>(w, h);
         U.load(((long long)(1 - hp.out_parity) * 4 + MU) * g.Vh + jb, u);
         const bool tm = MU == 3 && hp.chem;
-        transport_add<true, MU, -SF>(acc, u, h, tm ? f * hp.ebwd : f, SCALED || tm);
+        transport_add<true, MU, -SF>(accb ? accb : acc, u, h, tm ? f * hp.ebwd : f, SCALED || tm);
     }
 }
 
@@ -362,6 +364,7 @@ __device__ __forceinline__ void hop_staged(R* acc, const Field<P>& in, const Gau
 // and 8 for the plain loads) for memory-level parallelism per thread.
 
 constexpr int kPrefetchMinBlocks = 7;
+
 
 template <int T> struct TermOf {
     static constexpr int MU = T / 2;
@@ -639,18 +642,33 @@ template <int P> struct FuseArgs {
 // warps and blocks, which the CG scalars take, stay in FP64. Squares and
 // conversions in FP64 per element would put 48 FP64 instructions per thread
 // on a pipe that runs at 1/64 of the FP32 rate.
-template <typename A>
+template <bool SPLIT, typename A>
 __device__ __forceinline__ double block_sum128(A v, double* red) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int nthr = blockDim.x * blockDim.y;
+    const int tid = ((SPLIT ? threadIdx.z : 0) * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+    const int nthr = blockDim.x * blockDim.y * (SPLIT ? 4 : 1);
     if ((tid & 31) == 0) red[tid >> 5] = (double)v;
     __syncthreads();
     double tot = 0;
     if (tid == 0)
         for (int w = 0; w < (nthr + 31) / 32; ++w) tot += red[w];
     return tot;
+}
+
+// Adds the integer sums of the four threads (z) of a column into that of z = 0, through buf =
+// [z - 1][24][columns of the block]; every thread of the block takes part.
+__device__ __forceinline__ void join_terms(long long* v, long long* buf, int z, int tid) {
+    const int cols = blockDim.x * blockDim.y, col = tid - z * cols;
+    if (z > 0) {
+#pragma unroll
+        for (int k = 0; k < 24; ++k) buf[((z - 1) * 24 + k) * cols + col] = v[k];
+    }
+    __syncthreads();
+    if (z == 0) {
+#pragma unroll
+        for (int k = 0; k < 24; ++k) v[k] += (buf[k * cols + col] + buf[(24 + k) * cols + col]) + buf[(48 + k) * cols + col];
+    }
 }
 
 // shared memory of a hop block: [4 doubles: block reduction][2 mbarriers] then
@@ -676,13 +694,17 @@ constexpr bool kShuffleBidiag = MDWF_SHUFFLE_BIDIAG != 0;
 // launcher picks it when Ls matches), or -1 for the run-time choice; one
 // fixed length leaves the other lengths' code and its register demand out of
 // the kernel.
+// STAGE 5: a fourth of the thread block's columns, four threads (threadIdx.z = mu) per (site, s): each takes the two
+// terms of its direction, and their sums meet in shared memory. For lattices whose columns leave the SMs
+// with one block or less, where a hop takes as long as one thread's chain of eight neighbours (hop_shape).
 template <int P, bool DAG, bool XPAY, int FUSE, int STAGE, int LSR, bool DD = false>
 __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
+                                      : STAGE == 5 ? (P == MDWF_F64 ? 3 : 4)
                                       : STAGE == 3 ? kPrefetchMinBlocks
                                                    : PrecTraits<P>::min_blocks)
     hop_kernel(Field<P> out, Field<P> in, Field<P> xf, Gauge<P> U, HopParams<typename PrecTraits<P>::real> hp,
                FuseArgs<P> fa, FxArgs<P> fx) {
-    static_assert(!STAGE || P != MDWF_F64, "staged loads: FP32 / FP16 operators");
+    static_assert(!STAGE || STAGE == 5 || P != MDWF_F64, "staged loads: FP32 / FP16 operators");
     static_assert(!DD || (STAGE == 0 && FUSE == FUSE_NONE), "slab halos: plain loads, unfused");
     typedef typename PrecTraits<P>::real R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -696,7 +718,9 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     const int s = threadIdx.x, ly = threadIdx.y;
     const int rhs = blockIdx.x % hp.nrhs;
     const long long sblk = blockIdx.x / hp.nrhs;
-    const int tid = ly * blockDim.x + s, nthr = blockDim.x * blockDim.y;
+    const int z = STAGE == 5 ? threadIdx.z : 0;
+    const int tid = (z * blockDim.y + ly) * blockDim.x + s;
+    const int nthr = blockDim.x * blockDim.y * (STAGE == 5 ? 4 : 1);
     if (dense) {
         const R* gm = hp.mat + (size_t)rhs * 2 * Ls * Ls;
         for (int i = tid; i < 2 * Ls * Ls; i += nthr) mat[i] = gm[i];
@@ -706,7 +730,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         }
     }
     const long long site = sblk * blockDim.y + ly;
-    const bool active = site < hp.g.Vh;
+    const bool here = site < hp.g.Vh, active = here && z == 0;  // this thread's terms; this thread's epilogue
     const long long rbase = (long long)rhs * hp.g.Vh;
     const R mass = hp.mass[rhs];
     const SMass<R> sm{mass, hp.mass[kMaxRhs + rhs]};
@@ -716,7 +740,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     // backward ones at the neighbour), two lines per 80-byte FP32 link. The links and
     // the neighbour table do not change during a solve, so this runs before the wait
     // for the previous kernel.
-    if constexpr (P != MDWF_F64 && STAGE != 2) {
+    if constexpr (P != MDWF_F64 && STAGE != 2 && STAGE != 5) {
         if (active && s < 16) {
             const int* nbi = reinterpret_cast<const int*>(hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2);
             const int t = s >> 1, mu = t & 3;
@@ -733,7 +757,63 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     R acc[24];
 #pragma unroll
     for (int k = 0; k < 24; ++k) acc[k] = 0;
-    if constexpr (STAGE == 2) {
+    if constexpr (P == MDWF_F64 && !DD) {
+        const int* nbi = reinterpret_cast<const int*>(hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2);
+        long long sum[24];
+#pragma unroll
+        for (int k = 0; k < 24; ++k) sum[k] = 0;
+        int top = 0;
+        bool finite = true;
+        if (here)
+            finite = fx_terms<DAG, (STAGE == 5 ? 4 : 1)>(sum, top, z, fx, hp.g, hp.out_parity, nbi, site, s, rbase);
+        if constexpr (STAGE == 5) {
+            join_terms(sum, reinterpret_cast<long long*>(hs + (size_t)blockDim.y * site_stride(Ls)), z, tid);
+        }
+        if (active) {
+            if (finite) {
+                fx_finish(acc, sum, top);
+            } else {
+                double slow[24];
+                hop_nonfinite<DAG>(slow, fx.in, U, hp.g.Vh, hp.out_parity, hp.chem, hp.efwd, hp.ebwd, nbi, site, s,
+                                   rbase);
+#pragma unroll
+                for (int k = 0; k < 24; ++k) acc[k] = slow[k];
+            }
+        }
+    } else if constexpr (STAGE == 5) {
+        R back[24];
+#pragma unroll
+        for (int k = 0; k < 24; ++k) back[k] = 0;
+        if (here) {
+            const int* nbi = reinterpret_cast<const int*>(hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2);
+            switch (z) {
+                case 0: hop_dir<P, 0, DAG>(acc, in, U, hp, nbi, site, s, rbase, 0, back); break;
+                case 1: hop_dir<P, 1, DAG>(acc, in, U, hp, nbi, site, s, rbase, 0, back); break;
+                case 2: hop_dir<P, 2, DAG>(acc, in, U, hp, nbi, site, s, rbase, 0, back); break;
+                default: hop_dir<P, 3, DAG>(acc, in, U, hp, nbi, site, s, rbase, 0, back);
+            }
+        }
+        // the eight terms are added in the order of the other forms, which then give the same bits (FP16+norm would
+        // not: there the norm's product and the sum contract to one rounding)
+        R* buf = hs + (size_t)blockDim.y * site_stride(Ls);
+        const int cols = blockDim.x * blockDim.y, col = tid - z * cols;
+        if (z > 0) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k) {
+                buf[((z - 1) * 48 + k) * cols + col] = acc[k];
+                buf[((z - 1) * 48 + 24 + k) * cols + col] = back[k];
+            }
+        }
+        __syncthreads();
+        if (z == 0) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k) {
+                acc[k] += back[k];
+#pragma unroll
+                for (int t = 0; t < 6; ++t) acc[k] += buf[(t * 24 + k) * cols + col];
+            }
+        }
+    } else if constexpr (STAGE == 2) {
         // the buffers alias the rows of the epilogue (used after a barrier)
         Bulk<P> bk;
         bk.Ls = Ls;
@@ -747,16 +827,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         hop_bulk<P, DAG>(acc, in, U, hp, bk, bars, active, site, s, ly, tid, rbase);
     } else if (active) {
         const int4* nb = hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2;
-        if constexpr (P == MDWF_F64 && !DD) {
-            const int* nbi = reinterpret_cast<const int*>(nb);
-            if (!fx_hop<DAG>(acc, fx, hp.g, hp.out_parity, nbi, site, s, rbase)) {
-                double slow[24];
-                hop_nonfinite<DAG>(slow, fx.in, U, hp.g.Vh, hp.out_parity, hp.chem, hp.efwd, hp.ebwd, nbi, site, s,
-                                   rbase);
-#pragma unroll
-                for (int k = 0; k < 24; ++k) acc[k] = slow[k];
-            }
-        } else if constexpr (STAGE == 3) {
+        if constexpr (STAGE == 3) {
             hop_prefetch<P, DAG>(acc, in, U, hp, reinterpret_cast<const int*>(nb), site, s, rbase);
         } else if constexpr (STAGE == 1) {
             const int4 f = __ldg(nb), b = __ldg(nb + 1);
@@ -804,7 +875,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 #pragma unroll
             for (int k = 0; k < 24; ++k) y[k] = active ? fma(cf, acc[k], y[k]) : R(0);
             R* row = hs + (size_t)ly * site_stride(16) + s * kRowStride;
-            row_store(row, y);
+            if (z == 0) row_store(row, y);
             __syncthreads();
             const R sq = block_columns_a_adag<16>(hs, blockDim.y, hp.sc, sm, tid, nthr);
             __syncthreads();
@@ -812,7 +883,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
                 row_load(row, y);
                 fa.out2.store(rbase + site, s, y);
             }
-            const double tot = block_sum128(sq, red);
+            const double tot = block_sum128<STAGE == 5>(sq, red);
             if (tid == 0) fa.part[(size_t)rhs * (gridDim.x / hp.nrhs) + sblk] = tot;
             return;
         }
@@ -836,10 +907,10 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         shuffled = true;
     }
     if (!shuffled) {
-        row_store(mine, acc);
+        if (z == 0) row_store(mine, acc);
         __syncthreads();
         if (dense) {
-            dense_columns(mat, hs + (size_t)ly * sst, s, Ls, res);
+            if (z == 0) dense_columns(mat, hs + (size_t)ly * sst, s, Ls, res);
         } else {
             block_columns<LSR>(hs, blockDim.y, Ls, hp.sop, hp.swap != 0, hp.sc, sm, tid, nthr);
             __syncthreads();
@@ -894,10 +965,10 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 #pragma unroll
             for (int k = 0; k < 24; ++k) res[k] = R(0);
         }
-        row_store(mine, res);
+        if (z == 0) row_store(mine, res);
         __syncthreads();
         if (dense) {
-            dense_columns(mat2, hs + (size_t)ly * sst, s, Ls, res);
+            if (z == 0) dense_columns(mat2, hs + (size_t)ly * sst, s, Ls, res);
             if (active) store_hop(fa.out2, fx, rbase + site, s, res);
         } else {
             block_columns<LSR>(hs, blockDim.y, Ls, SOP_A, true, hp.sc, sm, tid, nthr);
@@ -922,7 +993,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             fa.rf.store(rbase + site, s, rv);
         }
     }
-    const double tot = block_sum128(sq, red);
+    const double tot = block_sum128<STAGE == 5>(sq, red);
     if (tid == 0) fa.part[(size_t)rhs * (gridDim.x / hp.nrhs) + sblk] = tot;
 }
 
@@ -932,13 +1003,14 @@ template <int P, bool D, bool X, int FU, int ST, int LSR, bool DD = false>
 static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<typename PrecTraits<P>::real>& hp) {
     typedef typename PrecTraits<P>::real R;
     const Geom& g = c->g;
-    const int SB = hop_sites_per_block(c, P, h.nrhs);
-    dim3 block(g.Ls, SB), grid((unsigned)((g.Vh + SB - 1) / SB * h.nrhs));
+    const int SB = hop_shape(c, P, h.nrhs).sites;
+    dim3 block(g.Ls, SB, ST == 5 ? 4 : 1), grid((unsigned)((g.Vh + SB - 1) / SB * h.nrhs));
     const size_t rows = (size_t)SB * site_stride(g.Ls) * sizeof(R);
     const size_t stage = ST == 1 ? (size_t)StageBytes<P>::value * g.Ls * SB
                          : ST == 2 ? (size_t)2 * BulkBytes<P>::value * g.Ls * SB : 0;
     const int ntab = hp.sop == SOP_DENSE ? (FU == FUSE_T ? 2 : 1) : 0;
-    size_t smem = kHopHeader + (size_t)ntab * 2 * g.Ls * g.Ls * sizeof(R) + (rows > stage ? rows : stage);
+    size_t smem = kHopHeader + (size_t)ntab * 2 * g.Ls * g.Ls * sizeof(R) + (rows > stage ? rows : stage) +
+                  (ST == 5 ? (size_t)3 * (P == MDWF_F64 ? 24 : 48) * g.Ls * SB * sizeof(R) : 0);
     auto kern = hop_kernel<P, D, X, FU, ST, LSR, DD>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1007,6 +1079,13 @@ static int launch_hop_pick(mdwf_ctx* c, const HopLaunch& h, const HopParams<type
         if (h.halo) return launch_hop_variant<P, D, X, FU, 0, -1, true>(c, h, hp);
     }
     if (h.halo) return MDWF_EINVAL;
+    if constexpr (P != MDWF_F16N) {
+        if (hop_shape(c, P, h.nrhs).split) {
+            if (P == MDWF_F32 && c->g.Ls == 16)
+                return launch_hop_variant<P, D, X, FU, 5, P == MDWF_F32 ? 16 : -1>(c, h, hp);
+            return launch_hop_variant<P, D, X, FU, 5, -1>(c, h, hp);
+        }
+    }
     if constexpr (P != MDWF_F64) {
         const int mode = c->hop_stage[P];
         if (mode == 1) return launch_hop_variant<P, D, X, FU, 1, -1>(c, h, hp);

@@ -978,6 +978,12 @@ int launch_hop(mdwf_ctx* c, int prec, const HopLaunch& h);
 // whether the fused CG iteration can run without its t field (HopLaunch::no_t)
 bool hop_no_t_ok(const mdwf_ctx* c, int prec, int nrhs);
 int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs);
+// the 4d sites per block of a hop launch, and whether four threads share each of its columns
+struct HopShape {
+    int sites;
+    bool split;
+};
+HopShape hop_shape(const mdwf_ctx* c, int prec, int nrhs);
 int hop_blocks(const mdwf_ctx* c, int prec, int nrhs);
 
 struct M5Launch {

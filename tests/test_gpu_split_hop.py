@@ -1,0 +1,52 @@
+"""The hop kernels with four threads per column (small lattices) against the ordinary block shape, which a tuned
+shape selects: the same bits in M, M^dag and the fused CG iterations."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import oracle
+import paper_1206_5214_gb300 as mdwf
+import synthetic as sy
+from _gpu import Ctx
+
+pytestmark = pytest.mark.gpu
+F64, F32 = mdwf.MDWF_F64, mdwf.MDWF_F32
+# the smallest field, columns that fill a warp, leave it ragged (10, 20, 24), exceed half of it, an odd last block
+SHAPES = [((2, 2, 2, 2), 2), ((4, 2, 2, 2), 8), ((6, 2, 2, 4), 10), ((4, 4, 2, 4), 16), ((2, 2, 2, 6), 16),
+          ((4, 2, 2, 4), 20), ((2, 4, 2, 4), 24), ((4, 2, 2, 2), 32)]
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("prec", [F64, F32])
+@pytest.mark.parametrize("dims,Ls", SHAPES)
+def test_apply_same_bits(dims, Ls, prec, dense):
+    U = sy.gauge_field(dims, 0.4, 1601)
+    odd = np.stack([oracle.split(sy.gaussian_field(dims, Ls, 2601 + r), dims)[1] for r in range(2)])
+    with Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.03, U, dense_s=dense) as c:
+        for dagger in (False, True):
+            split = c.apply(odd, prec, dagger, 2, [0.01, 0.2])
+            mdwf.mdwf_set_tuning(c.h, prec, 2, 128 // Ls)
+            plain = c.apply(odd, prec, dagger, 2, [0.01, 0.2])
+            mdwf.mdwf_set_tuning(c.h, prec, 2, 0)
+            assert np.array_equal(split, plain)
+
+
+@pytest.mark.parametrize("prec", [F64, F32])
+@pytest.mark.parametrize("dims,Ls", [((4, 4, 2, 4), 16), ((6, 2, 2, 4), 10), ((4, 2, 2, 4), 20)])
+def test_iterations_agree(dims, Ls, prec):
+    """Eight iterations of the fused CG: the vectors follow the same arithmetic, but the partial sums of the CG
+    scalars are grouped by block, so their last bits may differ (FP32 within a warp)."""
+    U = sy.gauge_field(dims, 0.4, 1602)
+    b = torch.from_numpy(sy.gaussian_field(dims, Ls, 2602)).cuda()
+    with Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.03, U) as c:
+        xs = []
+        for sites in (0, 128 // Ls):
+            mdwf.mdwf_set_tuning(c.h, prec, 1, sites)
+            x = torch.empty_like(b)
+            mdwf.mdwf_cgne(c.h, x, b, maxiter=8, inner_prec=prec, raise_on_error=False)
+            xs.append(x)
+        rel = float((xs[0] - xs[1]).norm() / xs[1].norm())
+    assert rel <= (1e-11 if prec == F64 else 1e-5), rel
