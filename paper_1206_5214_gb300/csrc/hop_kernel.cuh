@@ -555,7 +555,7 @@ __device__ __forceinline__ void hop_bulk(R* acc, const Field<P>& in, const Gauge
 //            residual field (precision PR) and the partial |r|^2 goes to part
 enum { FUSE_NONE = 0, FUSE_T = 1, FUSE_R = 2 };
 
-// The bidiagonal s-operators (M_phi = b5 + c5 C, C, I = M+ + M- C, and their
+// The bidiagonal s-operators 1 + w1 C (M_phi and I without their factors, and their
 // adjoints) for Ls = 16, where the 16 slices of a site fill one half-warp:
 // the s +- 1 neighbours of a column are lanes +- 1 of its 16-lane group, so
 // the column step needs shuffles and no shared memory. Chirality 0 (reals
@@ -563,18 +563,15 @@ enum { FUSE_NONE = 0, FUSE_T = 1, FUSE_R = 2 };
 // exchanges them; the wrap-around term carries -m. Every lane of the warp
 // must take part.
 template <typename R>
-__device__ __forceinline__ void bidiag_shuffle16(const R* in, R* out, int s, int op, bool swap, const SCoef<R>& sc,
-                                                 R m) {
-    bool w0;
-    R w1;
-    bidiag_weights(op, sc, w0, w1);
+__device__ __forceinline__ void bidiag_shuffle16(const R* in, R* out, int s, R w1, bool swap, R m) {
     const int up = (s + 1) & 15, dn = (s + 15) & 15;
     const int src0 = swap ? up : dn, src1 = swap ? dn : up;
     const R f0 = w1 * ((swap ? s < 15 : s > 0) ? R(1) : -m);
     const R f1 = w1 * ((swap ? s > 0 : s < 15) ? R(1) : -m);
 #pragma unroll
-    for (int k = 0; k < 24; ++k)
-        out[k] = fma(k < 12 ? f0 : f1, __shfl_sync(0xffffffffu, in[k], k < 12 ? src0 : src1, 16), w0 ? in[k] : R(0));
+    for (int k = 0; k < 12; ++k) out[k] = fma(f0, __shfl_sync(0xffffffffu, in[k], src0, 16), in[k]);
+#pragma unroll
+    for (int k = 12; k < 24; ++k) out[k] = fma(f1, __shfl_sync(0xffffffffu, in[k], src1, 16), in[k]);
 }
 
 // res = Mat col for the thread's slice s: Mat is the [chir][s'][s] table of one
@@ -871,7 +868,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 #pragma unroll
                 for (int k = 0; k < 24; ++k) xv[k] = R(0);
             }
-            bidiag_shuffle16(xv, y, s, SOP_MEE, false, hp.sc, mass);
+            bidiag_shuffle16(xv, y, s, hp.sc.r, false, mass);
 #pragma unroll
             for (int k = 0; k < 24; ++k) y[k] = active ? fma(cf, acc[k], y[k]) : R(0);
             R* row = hs + (size_t)ly * site_stride(16) + s * kRowStride;
@@ -896,8 +893,8 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     bool shuffled = false;
     if constexpr (LSR == 16) {
         if (kShuffleBidiag && !dense && (blockDim.y & 1) == 0 &&
-            (hp.sop == SOP_MPHI || hp.sop == SOP_C || hp.sop == SOP_MEE)) {
-            bidiag_shuffle16(acc, res, s, hp.sop, hp.swap != 0, hp.sc, mass);
+            ((hp.sop == SOP_MPHI && !hp.sc.b5_zero) || hp.sop == SOP_MEE)) {
+            bidiag_shuffle16(acc, res, s, hp.sop == SOP_MEE ? hp.sc.r : hp.sc.rho, hp.swap != 0, mass);
             shuffled = true;
         }
     }
@@ -932,7 +929,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 #pragma unroll
                 for (int k = 0; k < 24; ++k) xv[k] = R(0);
             }
-            bidiag_shuffle16(xv, tv, s, SOP_MEE, true, hp.sc, mass);
+            bidiag_shuffle16(xv, tv, s, hp.sc.r, true, mass);
 #pragma unroll
             for (int k = 0; k < 24; ++k) res[k] = fma(cf, res[k], tv[k]);
             xdone = true;

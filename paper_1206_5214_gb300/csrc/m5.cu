@@ -63,10 +63,18 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
             R h0[12], h1[12];
             in.load_half(sr, sw ? up : dn, 0, h0);
             in.load_half(sr, sw ? dn : up, 1, h1);
+            if (w0) {
 #pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                v[k] = fma(f0, h0[k], w0 ? v[k] : R(0));
-                v[12 + k] = fma(f1, h1[k], w0 ? v[12 + k] : R(0));
+                for (int k = 0; k < 12; ++k) {
+                    v[k] = fma(f0, h0[k], v[k]);
+                    v[12 + k] = fma(f1, h1[k], v[12 + k]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    v[k] = f0 * h0[k];
+                    v[12 + k] = f1 * h1[k];
+                }
             }
         }
         if (XPAY) {
