@@ -41,7 +41,8 @@ FLOPS_PER_SITE = 3120.0      # per odd 5d site and M (or M^dag) application
 # are now is stale and is not reported.
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_cgne_f32_16x16x16x32_Ls16.txt")
 KERNEL_SOURCES = ("paper_1206_5214_gb300/csrc/hop_kernel.cuh", "paper_1206_5214_gb300/csrc/mdwf_internal.cuh",
-                  "paper_1206_5214_gb300/csrc/mbarrier.cuh")
+                  "paper_1206_5214_gb300/csrc/mbarrier.cuh", "paper_1206_5214_gb300/csrc/spin.cuh",
+                  "paper_1206_5214_gb300/csrc/fx.cuh", "paper_1206_5214_gb300/csrc/fx_hop.cuh")
 METRIC = "Moebius Dslash GFLOP/s in CGNE to 1e-10 (mixed FP32/FP64)"
 # spectrum bounds of the Zolotarev coefficients of the per-slice solve: the upper one is
 # lambda_max = (8 - M5) / (10 - M5) of the Shamir kernel at M5 = 1.8 (Sec. 2)

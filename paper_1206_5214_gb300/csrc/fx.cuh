@@ -1,10 +1,14 @@
 // Fixed-point form of the FP64 hopping operator's operands, and the hopping sum on it.
 //
-// Why: GB300 issues 2 FP64 FMAs per clock and SM (measured 2.1) but 64 32x32+64-bit integer
-// multiply-adds (measured 61). The hopping sum of one 5d site is about 770 FP64 operations, which bound
-// the FP64 operator at 1.8 ms per hop on 16^3 x 32 x 16 with the memory nearly idle. Done on 64-bit
-// integers it is 1728 multiply-adds of 32-bit limbs and a few thousand cheap integer operations: 0.50 to 0.59 ms
-// per hop (the FP64 s-operators of the epilogue are then over half of it), M^dag 3.92 -> 1.36 ms.
+// Why: GB300 issues 2 FP64 FMAs per clock and SM (measured 2.1), but 32 products of two 32-bit integers with a
+// 64-bit result and 64 64-bit integer additions (the compiler makes one of each from a multiply-add). The hopping
+// sum of one 5d site is about 770 FP64 operations, which bound the FP64 operator at 1.8 ms per hop on 16^3 x 32 x 16
+// with the memory nearly idle. On 64-bit integers it is 1728 products and additions of 32-bit limbs and some
+// thousand cheap operations: 0.44 to 0.49 ms per hop with the s-operator of the epilogue, M 3.82 -> 1.00 ms, M^dag 3.92 ->
+// 1.08 ms. What bounds it now: about 8000 instructions per 5d site at 16 warps per SM (128 registers), issued on 42 %
+// of the cycles; the multiplier is 54 % busy, the FP64 pipe (s-operators) 32 %. One integer product of the upper
+// parts with FP32 cross terms needs a third of the products and was 5 % faster, but its error was above that of
+// FP64 in a quarter of the cases.
 //
 // Format: the 24 reals of one (site, s) spinor share a binary exponent e (the largest biased exponent
 // among them) and are stored as signed 64-bit integers q with value q 2^(e - 1080), |q| < 2^58. A link's
@@ -16,7 +20,8 @@
 // the largest of its eight neighbours' components, times a link entry of one, is 2^54 to 2^55 units.
 // FP64 arithmetic rounds every partial sum to 2^-53 of its size. M and M^dag against long double, 24 cases of
 // lattices, Ls, links and coefficients and four kinds of input (Gaussian, slices falling by e^-2, point
-// source, sites spread over decades): mean relative error 1.6e-16 in FP64, 1.3e-16 here; per site as well. Ranges: a neighbour's projected component is
+// source, sites spread over decades): mean relative error 1.62e-16 with FP64 hops, 1.26e-16 with these (and
+// 1.15e-16 with the s-operators as they are now); per site as well. Ranges: a neighbour's projected component is
 // below 2^59 (limbs |hi| <= 2^27, |lo| <= 2^31), so the middle sum is at most 6 (2^29 2^31 + 2^31 2^27) = 7.5
 // 2^60 < 2^63, a transported component at most 6 2^56, and the sum of eight terms at most 48 2^56 < 2^63.
 // Components more than 2^53 below the largest of their own spinor keep fewer bits than in FP64; each
