@@ -19,22 +19,23 @@ int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs) {
 }
 
 // The block shape of a hop launch. Where the whole s-columns of 128 threads make so few blocks that the time of a
-// hop is that of one thread's chain of eight neighbours, four threads share a column (STAGE 5 of the kernel). M alone,
-// ordinary and split form, by the number of ordinary blocks:
-//   FP32: 8 blocks 16.4 and 13.7 us, 128 blocks 17.0 and 14.4, 140 blocks 20.5 and 16.5, 256 blocks 16.5 and 20.5;
-//   FP64: 8 blocks 49 and 30 us, 32 blocks 51 and 33, 128 blocks 51 and 56, 256 blocks 65 and 96.
-// FP32 gains while the ordinary form leaves an SM at most one block; FP64, whose blocks wait for the integer
-// and FP64 pipes more than for memory, only while the four times as many split blocks still have an SM each.
+// hop is that of one thread's chain of eight neighbours, four or (FP64) two threads share a column (STAGE 5 and 6 of the
+// kernel). M alone in us, one, two and four threads a column, by the number of ordinary blocks:
+//   FP32: 8 blocks 16.4, -, 13.7; 128 blocks 17.0, -, 14.4; 140 blocks 20.5, -, 16.5; 256 blocks 16.5, -, 20.5
+//   FP64: 8 blocks 47, 34, 30; 64 blocks 49, 34, 34; 128 blocks 49, 43, 56; 205 blocks 64, 46, 72; 256 blocks 64, 77, 95
+// FP32 gains while the ordinary form leaves an SM at most one block. The FP64 split forms run three blocks per SM:
+// two threads a column pay while those blocks are one wave (205 blocks make 410, 256 make 512, of 456), four while
+// the integer pipe is not the limit.
 // Not for FP16+norm (its sums would round differently), a tuned block shape or a chosen load strategy.
-constexpr int kSplitBlocksF32 = 152, kSplitBlocksF64 = 152 / 4;
+constexpr int kSplit4BlocksF32 = 152, kSplit4BlocksF64 = 64, kSplit2BlocksF64 = 3 * 152 / 2;
 HopShape hop_shape(const mdwf_ctx* c, int prec, int nrhs) {
     const int sb = hop_sites_per_block(c, prec, nrhs);
     const long long blocks = (c->g.Vh + sb - 1) / sb * nrhs;
     const bool tuned = nrhs >= 1 && nrhs <= 64 && c->sb_tune[prec][nrhs] > 0;
-    if (prec == MDWF_F16N || c->slab || tuned || c->hop_stage[prec] != 0 || 
-        blocks > (prec == MDWF_F64 ? kSplitBlocksF64 : kSplitBlocksF32))
-        return {sb, false};
-    return {32 / c->g.Ls, true};
+    if (prec == MDWF_F16N || c->slab || tuned || c->hop_stage[prec] != 0) return {sb, 1};
+    if (blocks <= (prec == MDWF_F64 ? kSplit4BlocksF64 : kSplit4BlocksF32)) return {32 / c->g.Ls, 4};
+    if (prec == MDWF_F64 && blocks <= kSplit2BlocksF64) return {64 / c->g.Ls, 2};
+    return {sb, 1};
 }
 
 // The fused iteration drops its t field when the FUSE_R epilogue can rebuild

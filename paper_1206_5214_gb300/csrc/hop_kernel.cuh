@@ -364,6 +364,8 @@ __device__ __forceinline__ void hop_staged(R* acc, const Field<P>& in, const Gau
 // and 8 for the plain loads) for memory-level parallelism per thread.
 
 constexpr int kPrefetchMinBlocks = 7;
+// threads per (site, s) of a STAGE
+constexpr int split_of(int stage) { return stage == 5 ? 4 : stage == 6 ? 2 : 1; }
 
 
 template <int T> struct TermOf {
@@ -639,12 +641,12 @@ template <int P> struct FuseArgs {
 // warps and blocks, which the CG scalars take, stay in FP64. Squares and
 // conversions in FP64 per element would put 48 FP64 instructions per thread
 // on a pipe that runs at 1/64 of the FP32 rate.
-template <bool SPLIT, typename A>
+template <int Q, typename A>
 __device__ __forceinline__ double block_sum128(A v, double* red) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    const int tid = ((SPLIT ? threadIdx.z : 0) * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
-    const int nthr = blockDim.x * blockDim.y * (SPLIT ? 4 : 1);
+    const int tid = ((Q > 1 ? threadIdx.z : 0) * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+    const int nthr = blockDim.x * blockDim.y * Q;
     if ((tid & 31) == 0) red[tid >> 5] = (double)v;
     __syncthreads();
     double tot = 0;
@@ -653,8 +655,9 @@ __device__ __forceinline__ double block_sum128(A v, double* red) {
     return tot;
 }
 
-// Adds the integer sums of the four threads (z) of a column into that of z = 0, through buf =
+// Adds the integer sums of the Q threads (z) of a column into that of z = 0, through buf =
 // [z - 1][24][columns of the block]; every thread of the block takes part.
+template <int Q>
 __device__ __forceinline__ void join_terms(long long* v, long long* buf, int z, int tid) {
     const int cols = blockDim.x * blockDim.y, col = tid - z * cols;
     if (z > 0) {
@@ -664,7 +667,9 @@ __device__ __forceinline__ void join_terms(long long* v, long long* buf, int z, 
     __syncthreads();
     if (z == 0) {
 #pragma unroll
-        for (int k = 0; k < 24; ++k) v[k] += (buf[k * cols + col] + buf[(24 + k) * cols + col]) + buf[(48 + k) * cols + col];
+        for (int k = 0; k < 24; ++k)
+#pragma unroll
+            for (int t = 0; t < Q - 1; ++t) v[k] += buf[(t * 24 + k) * cols + col];
     }
 }
 
@@ -692,16 +697,17 @@ constexpr bool kShuffleBidiag = MDWF_SHUFFLE_BIDIAG != 0;
 // fixed length leaves the other lengths' code and its register demand out of
 // the kernel.
 // STAGE 5: a fourth of the thread block's columns, four threads (threadIdx.z = mu) per (site, s): each takes the two
-// terms of its direction, and their sums meet in shared memory. For lattices whose columns leave the SMs
+// terms of its direction, and their sums meet in shared memory. STAGE 6 (FP64): two threads with four terms each. For lattices whose columns leave the SMs
 // with one block or less, where a hop takes as long as one thread's chain of eight neighbours (hop_shape).
 template <int P, bool DAG, bool XPAY, int FUSE, int STAGE, int LSR, bool DD = false>
 __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
-                                      : STAGE == 5 ? (P == MDWF_F64 ? 3 : 4)
+                                      : STAGE >= 5 ? (P == MDWF_F64 ? 3 : 4)
                                       : STAGE == 3 ? kPrefetchMinBlocks
                                                    : PrecTraits<P>::min_blocks)
     hop_kernel(Field<P> out, Field<P> in, Field<P> xf, Gauge<P> U, HopParams<typename PrecTraits<P>::real> hp,
                FuseArgs<P> fa, FxArgs<P> fx) {
-    static_assert(!STAGE || STAGE == 5 || P != MDWF_F64, "staged loads: FP32 / FP16 operators");
+    static_assert(!STAGE || STAGE >= 5 || P != MDWF_F64, "staged loads: FP32 / FP16 operators");
+    constexpr int Q = split_of(STAGE);  // threads per (site, s)
     static_assert(!DD || (STAGE == 0 && FUSE == FUSE_NONE), "slab halos: plain loads, unfused");
     typedef typename PrecTraits<P>::real R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -715,9 +721,9 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     const int s = threadIdx.x, ly = threadIdx.y;
     const int rhs = blockIdx.x % hp.nrhs;
     const long long sblk = blockIdx.x / hp.nrhs;
-    const int z = STAGE == 5 ? threadIdx.z : 0;
+    const int z = Q > 1 ? threadIdx.z : 0;
     const int tid = (z * blockDim.y + ly) * blockDim.x + s;
-    const int nthr = blockDim.x * blockDim.y * (STAGE == 5 ? 4 : 1);
+    const int nthr = blockDim.x * blockDim.y * Q;
     if (dense) {
         const R* gm = hp.mat + (size_t)rhs * 2 * Ls * Ls;
         for (int i = tid; i < 2 * Ls * Ls; i += nthr) mat[i] = gm[i];
@@ -737,7 +743,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     // backward ones at the neighbour), two lines per 80-byte FP32 link. The links and
     // the neighbour table do not change during a solve, so this runs before the wait
     // for the previous kernel.
-    if constexpr (P != MDWF_F64 && STAGE != 2 && STAGE != 5) {
+    if constexpr (P != MDWF_F64 && STAGE != 2 && Q == 1) {
         if (active && s < 16) {
             const int* nbi = reinterpret_cast<const int*>(hp.nbr + ((long long)hp.out_parity * hp.g.Vh + site) * 2);
             const int t = s >> 1, mu = t & 3;
@@ -762,9 +768,9 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
         int top = 0;
         bool finite = true;
         if (here)
-            finite = fx_terms<DAG, (STAGE == 5 ? 4 : 1)>(sum, top, z, fx, hp.g, hp.out_parity, nbi, site, s, rbase);
-        if constexpr (STAGE == 5) {
-            join_terms(sum, reinterpret_cast<long long*>(hs + (size_t)blockDim.y * site_stride(Ls)), z, tid);
+            finite = fx_terms<DAG, Q>(sum, top, z, fx, hp.g, hp.out_parity, nbi, site, s, rbase);
+        if constexpr (Q > 1) {
+            join_terms<Q>(sum, reinterpret_cast<long long*>(hs + (size_t)blockDim.y * site_stride(Ls)), z, tid);
         }
         if (active) {
             if (finite) {
@@ -880,7 +886,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
                 row_load(row, y);
                 fa.out2.store(rbase + site, s, y);
             }
-            const double tot = block_sum128<STAGE == 5>(sq, red);
+            const double tot = block_sum128<Q>(sq, red);
             if (tid == 0) fa.part[(size_t)rhs * (gridDim.x / hp.nrhs) + sblk] = tot;
             return;
         }
@@ -893,7 +899,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
     bool shuffled = false;
     if constexpr (LSR == 16) {
         if (kShuffleBidiag && !dense && (blockDim.y & 1) == 0 &&
-            ((hp.sop == SOP_MPHI && !hp.sc.b5_zero) || hp.sop == SOP_MEE)) {
+            ((hp.sop == SOP_MPHI && !hp.sc.raw) || hp.sop == SOP_MEE)) {
             bidiag_shuffle16(acc, res, s, hp.sop == SOP_MEE ? hp.sc.r : hp.sc.rho, hp.swap != 0, mass);
             shuffled = true;
         }
@@ -990,7 +996,7 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
             fa.rf.store(rbase + site, s, rv);
         }
     }
-    const double tot = block_sum128<STAGE == 5>(sq, red);
+    const double tot = block_sum128<Q>(sq, red);
     if (tid == 0) fa.part[(size_t)rhs * (gridDim.x / hp.nrhs) + sblk] = tot;
 }
 
@@ -1001,13 +1007,13 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
     typedef typename PrecTraits<P>::real R;
     const Geom& g = c->g;
     const int SB = hop_shape(c, P, h.nrhs).sites;
-    dim3 block(g.Ls, SB, ST == 5 ? 4 : 1), grid((unsigned)((g.Vh + SB - 1) / SB * h.nrhs));
+    dim3 block(g.Ls, SB, split_of(ST)), grid((unsigned)((g.Vh + SB - 1) / SB * h.nrhs));
     const size_t rows = (size_t)SB * site_stride(g.Ls) * sizeof(R);
     const size_t stage = ST == 1 ? (size_t)StageBytes<P>::value * g.Ls * SB
                          : ST == 2 ? (size_t)2 * BulkBytes<P>::value * g.Ls * SB : 0;
     const int ntab = hp.sop == SOP_DENSE ? (FU == FUSE_T ? 2 : 1) : 0;
     size_t smem = kHopHeader + (size_t)ntab * 2 * g.Ls * g.Ls * sizeof(R) + (rows > stage ? rows : stage) +
-                  (ST == 5 ? (size_t)3 * (P == MDWF_F64 ? 24 : 48) * g.Ls * SB * sizeof(R) : 0);
+                  (size_t)(split_of(ST) - 1) * (P == MDWF_F64 ? 24 : 48) * g.Ls * SB * sizeof(R);
     auto kern = hop_kernel<P, D, X, FU, ST, LSR, DD>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1076,12 +1082,15 @@ static int launch_hop_pick(mdwf_ctx* c, const HopLaunch& h, const HopParams<type
         if (h.halo) return launch_hop_variant<P, D, X, FU, 0, -1, true>(c, h, hp);
     }
     if (h.halo) return MDWF_EINVAL;
-    if constexpr (P != MDWF_F16N) {
-        if (hop_shape(c, P, h.nrhs).split) {
-            if (P == MDWF_F32 && c->g.Ls == 16)
-                return launch_hop_variant<P, D, X, FU, 5, P == MDWF_F32 ? 16 : -1>(c, h, hp);
-            return launch_hop_variant<P, D, X, FU, 5, -1>(c, h, hp);
-        }
+    const int split = hop_shape(c, P, h.nrhs).split;
+    if constexpr (P == MDWF_F32) {
+        if (split == 4)
+            return c->g.Ls == 16 ? launch_hop_variant<P, D, X, FU, 5, 16>(c, h, hp)
+                                 : launch_hop_variant<P, D, X, FU, 5, -1>(c, h, hp);
+    }
+    if constexpr (P == MDWF_F64) {
+        if (split == 4) return launch_hop_variant<P, D, X, FU, 5, -1>(c, h, hp);
+        if (split == 2) return launch_hop_variant<P, D, X, FU, 6, -1>(c, h, hp);
     }
     if constexpr (P != MDWF_F64) {
         const int mode = c->hop_stage[P];

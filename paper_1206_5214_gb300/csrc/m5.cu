@@ -52,8 +52,7 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
         R v[24];
         in.load(sr, s, v);
         if (bidiag) {
-            bool w0;
-            R w1;
+            R w0, w1;
             bidiag_weights(sop, sc, w0, w1);
             const R m = mass[rhs];
             const bool sw = swap != 0;
@@ -63,7 +62,7 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
             R h0[12], h1[12];
             in.load_half(sr, sw ? up : dn, 0, h0);
             in.load_half(sr, sw ? dn : up, 1, h1);
-            if (w0) {
+            if (w0 == R(1)) {
 #pragma unroll
                 for (int k = 0; k < 12; ++k) {
                     v[k] = fma(f0, h0[k], v[k]);
@@ -72,8 +71,8 @@ __global__ void __launch_bounds__(256) m5_kernel(Field<P> out, Field<P> in, Fiel
             } else {
 #pragma unroll
                 for (int k = 0; k < 12; ++k) {
-                    v[k] = f0 * h0[k];
-                    v[12 + k] = f1 * h1[k];
+                    v[k] = fma(f0, h0[k], w0 * v[k]);
+                    v[12 + k] = fma(f1, h1[k], w0 * v[12 + k]);
                 }
             }
         }

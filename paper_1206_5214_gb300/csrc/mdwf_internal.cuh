@@ -18,6 +18,7 @@
 #pragma once
 
 #include <cuda_fp16.h>
+#include <math.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -450,12 +451,13 @@ enum SOp { SOP_DENSE = 0, SOP_ID = 1, SOP_A = 2, SOP_MPHI = 3, SOP_K = 4, SOP_C 
 //        Psi_s = b_s - r Psi_{s+1}
 //   K~:  (K~ b)_s = Psi_s + rho Psi_{s+1} = b_s + (rho - r) Psi_{s+1},  (K~ b)_{Ls-1} = Psi_{Ls-1} - m rho Psi_0,
 // two and three multiply-adds per real (A: 3.5 operations and a division per column before, K: 5.5). In FP64 this is
-// what the hop epilogues cost: 2 FMAs per clock and SM. With b5 = 0, M_phi and K keep their factor (c5 C, c5 C A).
+// what the hop epilogues cost: 2 FMAs per clock and SM. Where b5 is zero or small beside c5 (below 1e-3 |c5|, rho could
+// overflow), M_phi and K keep their factor (`raw`: b5 + c5 C as it stands).
 // q depends on the mass and is computed on the host ([kMaxRhs] masses, then [kMaxRhs] values of q).
 template <typename R> struct SCoef {
-    R c5, r, rho, krho;  // krho = rho - r
-    R inv;               // 1 / M+ (K with b5 = 0)
-    int b5_zero;
+    R r, rho, krho;      // krho = rho - r
+    int raw;
+    R b5, c5, inv;       // raw M_phi and K; inv = 1 / M+
     R rp[kMaxLs];        // (-r)^s
 };
 template <typename R> struct SMass {
@@ -467,11 +469,11 @@ template <typename R> struct CPair;
 template <> struct CPair<float> { typedef float2 T; };
 template <> struct CPair<double> { typedef double2 T; };
 
-// The weights (w0, w1) of a bidiagonal operator w0 + w1 C.
+// The weights of a bidiagonal operator w0 + w1 C (w0 is 1 except for C and raw M_phi).
 template <typename R>
-__device__ __forceinline__ void bidiag_weights(int op, const SCoef<R>& sc, bool& w0, R& w1) {
-    w0 = op == SOP_MEE || (op == SOP_MPHI && !sc.b5_zero);
-    w1 = op == SOP_MEE ? sc.r : op == SOP_MPHI ? (sc.b5_zero ? sc.c5 : sc.rho) : R(1);
+__device__ __forceinline__ void bidiag_weights(int op, const SCoef<R>& sc, R& w0, R& w1) {
+    w0 = op == SOP_MEE ? R(1) : op == SOP_MPHI ? (sc.raw ? sc.b5 : R(1)) : R(0);
+    w1 = op == SOP_MEE ? sc.r : op == SOP_MPHI ? (sc.raw ? sc.c5 : sc.rho) : R(1);
 }
 
 // In place on one complex column: element s at base[k(s) * stride] (re, im as
@@ -508,40 +510,44 @@ __device__ __forceinline__ void column_op(R* base, int stride, int Ls, int op, b
                 C* t = at(s);
                 const C b = *t;
                 C o;
-                if (sc.b5_zero) {
-                    o.x = sc.c5 * (sc.inv * pr);
-                    o.y = sc.c5 * (sc.inv * pi);
+                const R nr = fma(-r, pr, b.x), ni = fma(-r, pi, b.y);  // Psi_s
+                if (sc.raw) {
+                    o.x = sc.inv * fma(sc.c5, pr, sc.b5 * nr);
+                    o.y = sc.inv * fma(sc.c5, pi, sc.b5 * ni);
                 } else {
                     o.x = fma(sc.krho, pr, b.x);
                     o.y = fma(sc.krho, pi, b.y);
                 }
                 *t = o;
-                pr = fma(-r, pr, b.x);
-                pi = fma(-r, pi, b.y);
+                pr = nr;
+                pi = ni;
             }
             C o;  // row Ls-1 wraps to Psi_0 (now in pr, pi) with -m
-            const R w = -sm.m * (sc.b5_zero ? sc.c5 * sc.inv : sc.rho);
-            o.x = fma(w, pr, sc.b5_zero ? R(0) : lr);
-            o.y = fma(w, pi, sc.b5_zero ? R(0) : li);
+            if (sc.raw) {
+                o.x = sc.inv * fma(-sm.m * sc.c5, pr, sc.b5 * lr);
+                o.y = sc.inv * fma(-sm.m * sc.c5, pi, sc.b5 * li);
+            } else {
+                o.x = fma(-sm.m * sc.rho, pr, lr);
+                o.y = fma(-sm.m * sc.rho, pi, li);
+            }
             *at(Ls - 1) = o;
         }
     } else if (op == SOP_MPHI || op == SOP_C || op == SOP_MEE) {
-        bool w0;
-        R w1;
+        R w0, w1;
         bidiag_weights(op, sc, w0, w1);
         const C f0 = *at(0);
         C cur = f0;
         for (int s = 0; s < Ls - 1; ++s) {
             const C nxt = *at(s + 1);
             C o;
-            o.x = fma(w1, nxt.x, w0 ? cur.x : R(0));
-            o.y = fma(w1, nxt.y, w0 ? cur.y : R(0));
+            o.x = fma(w1, nxt.x, w0 == R(1) ? cur.x : w0 * cur.x);
+            o.y = fma(w1, nxt.y, w0 == R(1) ? cur.y : w0 * cur.y);
             *at(s) = o;
             cur = nxt;
         }
         C o;
-        o.x = fma(-sm.m * w1, f0.x, w0 ? cur.x : R(0));
-        o.y = fma(-sm.m * w1, f0.y, w0 ? cur.y : R(0));
+        o.x = fma(-sm.m * w1, f0.x, w0 == R(1) ? cur.x : w0 * cur.x);
+        o.y = fma(-sm.m * w1, f0.y, w0 == R(1) ? cur.y : w0 * cur.y);
         *at(Ls - 1) = o;
     }
 }
@@ -579,13 +585,13 @@ __device__ __forceinline__ void a_solve(C* v, const SCoef<R>& sc, const SMass<R>
 
 // column_op with the column held in registers (Ls known at compile time): all
 // Ls elements are loaded at once, the recursion runs on registers, and all are
-// stored back; the arithmetic is that of column_op. (C, and with b5 = 0 M_phi and K,
-// which no tuned path uses, go through column_op.)
+// stored back; the arithmetic is that of column_op. (C and the raw M_phi and K, which no
+// tuned path uses, go through column_op.)
 template <int LS, typename R>
 __device__ __forceinline__ void column_op_reg(R* base, int stride, int op, bool up, const SCoef<R>& sc,
                                               const SMass<R>& sm) {
     typedef typename CPair<R>::T C;
-    if (op == SOP_C || (sc.b5_zero && (op == SOP_K || op == SOP_MPHI))) {
+    if (op == SOP_C || (sc.raw && (op == SOP_K || op == SOP_MPHI))) {
         column_op(base, stride, LS, op, up, sc, sm);
         return;
     }
@@ -901,16 +907,18 @@ template <class L> inline void set_sop(const mdwf_ctx* c, int prec, int sop, int
     }
 }
 
+// Whether M_phi and K keep their factor (SCoef::raw).
+inline bool mphi_raw(const mdwf_ctx* c) { return !(fabs(c->b5) >= 1e-3 * fabs(c->c5)) || c->b5 == 0.0; }
 // The constant factor that a launch of s-operator sop leaves out (SCoef); 1 for dense tables.
 inline double sop_scale(const mdwf_ctx* c, int sop) {
     if (sop == SOP_DENSE) return 1.0;
     const double Mp = c->b5 * (4.0 - c->M5) + 1.0;
-    const bool z = c->b5 == 0.0;
+    const bool raw = mphi_raw(c);
     switch (sop) {
         case SOP_A: return 1.0 / Mp;
         case SOP_MEE: return Mp;
-        case SOP_MPHI: return z ? 1.0 : c->b5;
-        case SOP_K: return z ? 1.0 : c->b5 / Mp;
+        case SOP_MPHI: return raw ? 1.0 : c->b5;
+        case SOP_K: return raw ? 1.0 : c->b5 / Mp;
     }
     return 1.0;
 }
@@ -920,13 +928,14 @@ inline double ctx_scale(const mdwf_ctx* c, int sop) { return c->dense_s ? 1.0 : 
 template <typename R> inline SCoef<R> make_scoef(const mdwf_ctx* c) {
     SCoef<R> sc;
     const double Mp = c->b5 * (4.0 - c->M5) + 1.0, Mm = c->c5 * (4.0 - c->M5) - 1.0;
-    const double r = Mp != 0.0 ? Mm / Mp : 0.0, rho = c->b5 != 0.0 ? c->c5 / c->b5 : 0.0;
+    const double r = Mp != 0.0 ? Mm / Mp : 0.0, rho = mphi_raw(c) ? 0.0 : c->c5 / c->b5;
+    sc.b5 = (R)c->b5;
     sc.c5 = (R)c->c5;
     sc.r = (R)r;
     sc.rho = (R)rho;
     sc.krho = (R)(rho - r);
     sc.inv = (R)(Mp != 0.0 ? 1.0 / Mp : 0.0);
-    sc.b5_zero = c->b5 == 0.0;
+    sc.raw = mphi_raw(c);
     double pw = 1.0;
     for (int s = 0; s < kMaxLs; ++s, pw *= -r) sc.rp[s] = (R)pw;
     return sc;
@@ -978,10 +987,9 @@ int launch_hop(mdwf_ctx* c, int prec, const HopLaunch& h);
 // whether the fused CG iteration can run without its t field (HopLaunch::no_t)
 bool hop_no_t_ok(const mdwf_ctx* c, int prec, int nrhs);
 int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs);
-// the 4d sites per block of a hop launch, and whether four threads share each of its columns
+// the 4d sites per block of a hop launch, and how many threads share each of its columns
 struct HopShape {
-    int sites;
-    bool split;
+    int sites, split;
 };
 HopShape hop_shape(const mdwf_ctx* c, int prec, int nrhs);
 int hop_blocks(const mdwf_ctx* c, int prec, int nrhs);

@@ -1,4 +1,4 @@
-"""The hop kernels with four threads per column (small lattices) against the ordinary block shape, which a tuned
+"""The hop kernels with four or two threads per column (small lattices) against the ordinary block shape, which a tuned
 shape selects: the same bits in M, M^dag and the fused CG iterations."""
 import numpy as np
 import pytest
@@ -16,7 +16,9 @@ pytestmark = pytest.mark.gpu
 F64, F32 = mdwf.MDWF_F64, mdwf.MDWF_F32
 # the smallest field, columns that fill a warp, leave it ragged (10, 20, 24), exceed half of it, an odd last block
 SHAPES = [((2, 2, 2, 2), 2), ((4, 2, 2, 2), 8), ((6, 2, 2, 4), 10), ((4, 4, 2, 4), 16), ((2, 2, 2, 6), 16),
-          ((4, 2, 2, 4), 20), ((2, 4, 2, 4), 24), ((4, 2, 2, 2), 32)]
+          ((4, 2, 2, 4), 20), ((2, 4, 2, 4), 24), ((4, 2, 2, 2), 32),
+          # FP64 with two threads: 65 to 228 ordinary blocks
+          ((8, 8, 4, 8), 10), ((4, 4, 6, 8), 24), ((4, 4, 4, 10), 32), ((8, 8, 8, 4), 16)]
 
 
 @pytest.mark.parametrize("dense", [False, True])
@@ -35,7 +37,7 @@ def test_apply_same_bits(dims, Ls, prec, dense):
 
 
 @pytest.mark.parametrize("prec", [F64, F32])
-@pytest.mark.parametrize("dims,Ls", [((4, 4, 2, 4), 16), ((6, 2, 2, 4), 10), ((4, 2, 2, 4), 20)])
+@pytest.mark.parametrize("dims,Ls", [((4, 4, 2, 4), 16), ((6, 2, 2, 4), 10), ((4, 2, 2, 4), 20), ((4, 4, 6, 8), 24)])
 def test_iterations_agree(dims, Ls, prec):
     """Eight iterations of the fused CG: the vectors follow the same arithmetic, but the partial sums of the CG
     scalars are grouped by block, so their last bits may differ (FP32 within a warp)."""
