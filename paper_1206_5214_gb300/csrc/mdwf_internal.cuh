@@ -788,9 +788,9 @@ struct mdwf_ctx {
     mdwf::Geom g{};
     double M5 = 0, b5 = 0, c5 = 0, mf = 0;
     bool have_gauge = false;
-    void* gauge[2] = {nullptr, nullptr};  // FP64 and FP32 copies
-    void* gauge_fx = nullptr;             // fixed-point copy (fx.cuh), 144 B per link as the FP64 one
-    int* gauge_fx_exp = nullptr;          // and its exponents, behind it in the same allocation
+    void* gauge[2] = {nullptr, nullptr};  // FP64 and FP32 copies, in one allocation with
+    void* gauge_fx = nullptr;             // the fixed-point copy (fx.cuh), 144 B per link as the FP64 one,
+    int* gauge_fx_exp = nullptr;          // and its exponents
     // Ls x Ls tables for the current mass list, FP64 and FP32, plus per-rhs masses
     double* tab64 = nullptr;
     float* tab32 = nullptr;
