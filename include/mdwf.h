@@ -200,7 +200,8 @@ int mdwf_get_s_coefficients(const mdwf_ctx *ctx, double *b5s, double *c5s, int *
  * Loads the SU(3) links U_mu(x) (Eq. D^Wilson) from complex128
  * U[t][z][y][x][mu][3][3] in host (where = MDWF_HOST) or device memory.
  * The data is copied into per-parity, per-direction link arrays in FP64 and
- * FP32 (the FP32 copy also serves the FP16+norm operator); the caller's buffer
+ * FP32 (the FP32 copy also serves the FP16+norm operator), and for the FP64
+ * hops in 64-bit fixed point (not on t-slabs); the caller's buffer
  * may be reused once the call returns (host) or once the stream has passed
  * this point (device).
  */
@@ -264,7 +265,7 @@ typedef struct {
                              with FP64 reliable updates of x and the true residual */
     double delta;         /* reliable-update threshold on |r| / max |r|; 0 = 0.005 (FP32 inner), 0.1 (FP16N) */
     int check_every;      /* iterations between host convergence polls; 0 = 8 */
-    int use_graph;        /* 1: replay the CG iteration as a captured CUDA graph */
+    int use_graph;        /* 1: replay the CG iterations as captured CUDA graphs */
     int guess;            /* 1: x holds an initial guess on entry and the CG starts from its odd
                              part (a restart or warm start); 0: the CG starts from zero */
 } mdwf_solve_params;
