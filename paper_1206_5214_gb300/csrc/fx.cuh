@@ -24,23 +24,34 @@
 // 1.15e-16 with the s-operators as they are now); per site as well. Ranges: a neighbour's projected component is
 // below 2^59 (limbs |hi| <= 2^27, |lo| <= 2^31), so the middle sum is at most 6 (2^29 2^31 + 2^31 2^27) = 7.5
 // 2^60 < 2^63, a transported component at most 6 2^56, and the sum of eight terms at most 48 2^56 < 2^63.
-// Components more than 2^53 below the largest of their own spinor keep fewer bits than in FP64; each
-// is mixed with that component by the link and the spin projection that follow.
 //
-// Non-finite spinors are stored as the raw doubles with exponent kFxRaw, and a site that has such a
-// neighbour (or link) takes the FP64 arithmetic, so that infinities and NaN spread as there.
+// Small parts beside large ones: the error above is relative to the largest component that reaches a site, where
+// FP64 arithmetic errs relative to what each component is made of. The two differ where parts of the field do not
+// mix: a hopping term adds to an upper spin only that spin and the lower ones (and the reverse), and links
+// diagonal in colour (a free field) keep the colours apart. So a spinor is stored in fixed point only if in every
+// colour each spin, together with the two of the other chirality, reaches 2^-kFxSpread of the largest component, and a
+// link only if its rows and columns do; others (point sources, fields of one colour) are kept as raw doubles. The terms
+// of a component then add up to 2^(54 - kFxSpread) units times a link entry of 0.4, 2^46, or more, and 8 terms
+// are off by 32 units at most and by 1.5 in the root mean square: 2^-41 and 2^-45 of the component at the very
+// edge of the rule, FP64's accuracy away from it.
+// Gaussian fields cross the line at one spinor in 10^10. Fields of one chirality alone cross it at one in 600, and
+// a warp reads 256: M on 16^3 x 32 x 16 then takes 2.2 ms, 2.2 for one colour, 1.01 otherwise (1.006 without the rule;
+// 3.8 in FP64 arithmetic). kFxSpread = 5 takes 3.4 ms there and the FP64 solve on 8^3 x 16 x 12 79 instead of 64 ms;
+// 10 takes 1.07 for one chirality. In solves the chiralities stay within a factor of 1.2 of each other.
+//
+// Raw spinors and links carry the exponent kFxRaw, and a site that has such a neighbour (or link) takes the FP64
+// arithmetic; non-finite ones are stored so too, so that infinities and NaN spread as there.
 #pragma once
 
 #include "mdwf_internal.cuh"
 
 namespace mdwf {
 
-template <int V> struct IntC { static constexpr int value = V; };
-
 constexpr int kFxFieldBias = 1080, kFxLinkBias = 1083;
 constexpr int kFxZero = -(1 << 20);   // exponent of an all-zero spinor or link
-constexpr int kFxRaw = 1 << 24;       // exponent of a spinor or link with a non-finite entry
+constexpr int kFxRaw = 1 << 24;       // exponent of a spinor or link kept as doubles
 constexpr int kFxRawMin = 1 << 22;    // sums of exponents at or above this hold a kFxRaw
+constexpr int kFxSpread = 7;          // binary orders between the parts of a fixed-point spinor or link
 
 // shared exponent of n doubles: the largest biased exponent, kFxZero or kFxRaw
 template <int N>
@@ -55,6 +66,37 @@ __device__ __forceinline__ int fx_exponent(const double* v) {
     if (e == 0x7ff) return kFxRaw;
     if (m == 0 && low == 0) return kFxZero;
     return max(e, 1);  // subnormals carry the exponent 1
+}
+
+// the upper word of |v|: sizes compare by it to within a factor of two
+__device__ __forceinline__ int fx_size(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// whether a spinor's parts are close enough in size for one exponent (the rule above); false for parts that are zero
+__device__ __forceinline__ bool fx_spinor_even(const double* v) {
+    int top = 0, low = 0x7fffffff;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        int a[4];  // the four spins
+#pragma unroll
+        for (int b = 0; b < 4; ++b) a[b] = max(fx_size(v[6 * b + 2 * c]), fx_size(v[6 * b + 2 * c + 1]));
+        const int u = max(a[0], a[1]), l = max(a[2], a[3]);
+        low = min(low, min(max(min(a[0], a[1]), l), max(min(a[2], a[3]), u)));
+        top = max(top, max(u, l));
+    }
+    return low >= top - (kFxSpread << 20);
+}
+
+// the same for the rows and columns of a link
+__device__ __forceinline__ bool fx_link_even(const double* v) {
+    int row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int a = max(fx_size(v[2 * k]), fx_size(v[2 * k + 1]));
+        row[k / 3] = max(row[k / 3], a);
+        col[k % 3] = max(col[k % 3], a);
+    }
+    const int top = max(row[0], max(row[1], row[2]));
+    return min(min(row[0], min(row[1], row[2])), min(col[0], min(col[1], col[2]))) >= top - (kFxSpread << 20);
 }
 
 // v as an integer at the shared exponent e, with SH guard bits below the 53 of a double (truncated)
@@ -107,20 +149,28 @@ struct FxField {
             o[2 * k + 1] = d.y;
         }
     }
-    // the spinor as doubles (the path of non-finite neighbours)
+    // the spinor as doubles, exactly (the path of raw neighbours)
     __device__ __forceinline__ void load(long long sr, int s, double* o) const {
         long long q[24];
         load(sr, s, q);
-        const int x = exponent(sr, s);
-        for (int k = 0; k < 24; ++k)
-            o[k] = x == kFxRaw ? __longlong_as_double(q[k]) : x == kFxZero ? 0.0 : scalbn((double)q[k], x - kFxFieldBias);
+        const int e = exponent(sr, s), x = e - kFxFieldBias;
+        if (e == kFxRaw) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k) o[k] = __longlong_as_double(q[k]);
+        } else if (fx_scale_safe(x)) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k) o[k] = fx_to_double(q[k], x);
+        } else {
+            for (int k = 0; k < 24; ++k) o[k] = e == kFxZero ? 0.0 : scalbn((double)q[k], x);
+        }
     }
 };
 
 // writes a spinor of doubles in fixed point
 __device__ __forceinline__ void fx_store(const Field<MDWF_F64>& f, int* e, long long sr, int s, const double* v) {
     if (f.bnd.bad(sr, s, f.Ls)) return;
-    const int x = fx_exponent<24>(v);
+    int x = fx_exponent<24>(v);
+    if (x != kFxZero && !fx_spinor_even(v)) x = kFxRaw;
     longlong2* p = reinterpret_cast<longlong2*>(f.v) + sr * 12 * f.Ls + s;
     if (x == kFxRaw) {
 #pragma unroll

@@ -100,8 +100,8 @@ struct FxHop {
 };
 
 // Terms t0, t0 + DT, ... of the eight of one (site, s), t = 0..3 the forward ones, 4..7 the backward ones: their sum
-// as integers at the exponent `top` of the largest term of all eight. False where a neighbour or a link is not
-// finite (the caller then takes the FP64 arithmetic).
+// as integers at the exponent `top` of the largest term of all eight. False where a neighbour or a link is
+// raw (the caller then takes the FP64 arithmetic).
 template <bool DAG, int DT>
 __device__ __forceinline__ bool fx_terms(long long* acc, int& top, int t0, const FxHop& fx, const Geom& g,
                                          int out_parity, const int* nbi, long long site, int s, long long rbase) {

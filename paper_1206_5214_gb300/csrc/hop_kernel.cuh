@@ -599,9 +599,9 @@ template <int P> struct ResPrec { static constexpr int value = P == MDWF_F64 ? M
 template <int P> struct FxArgs {};
 template <> struct FxArgs<MDWF_F64> : FxHop {};
 
-// The FP64 arithmetic for a site with a non-finite neighbour or link (rare: not inlined).
+// The FP64 arithmetic for a site with a raw neighbour or link (rare: not inlined).
 template <bool DAG>
-__device__ __noinline__ void hop_nonfinite(double* acc, FxField in, Gauge<MDWF_F64> U, long long Vh, int out_parity,
+__device__ __noinline__ void hop_raw(double* acc, FxField in, Gauge<MDWF_F64> U, long long Vh, int out_parity,
                                            bool chem, double efwd, double ebwd, const int* nbi, long long site, int s,
                                            long long rbase) {
     HopParams<double> hp;
@@ -766,19 +766,18 @@ __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
 #pragma unroll
         for (int k = 0; k < 24; ++k) sum[k] = 0;
         int top = 0;
-        bool finite = true;
+        bool fixed = true;
         if (here)
-            finite = fx_terms<DAG, Q>(sum, top, z, fx, hp.g, hp.out_parity, nbi, site, s, rbase);
+            fixed = fx_terms<DAG, Q>(sum, top, z, fx, hp.g, hp.out_parity, nbi, site, s, rbase);
         if constexpr (Q > 1) {
             join_terms<Q>(sum, reinterpret_cast<long long*>(hs + (size_t)blockDim.y * site_stride(Ls)), z, tid);
         }
         if (active) {
-            if (finite) {
+            if (fixed) {
                 fx_finish(acc, sum, top);
             } else {
                 double slow[24];
-                hop_nonfinite<DAG>(slow, fx.in, U, hp.g.Vh, hp.out_parity, hp.chem, hp.efwd, hp.ebwd, nbi, site, s,
-                                   rbase);
+                hop_raw<DAG>(slow, fx.in, U, hp.g.Vh, hp.out_parity, hp.chem, hp.efwd, hp.ebwd, nbi, site, s, rbase);
 #pragma unroll
                 for (int k = 0; k < 24; ++k) acc[k] = slow[k];
             }

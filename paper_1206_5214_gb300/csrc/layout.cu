@@ -115,7 +115,8 @@ __global__ void gauge_pack_kernel(double2* u64, float* u32, int4* fx, int* fx_ex
                 v[2 * k] = src[k].x;
                 v[2 * k + 1] = src[k].y;
             }
-            const int e = fx_exponent<18>(v);
+            int e = fx_exponent<18>(v);
+            if (e != kFxZero && !fx_link_even(v)) e = kFxRaw;
             fx_exp[l] = e;
 #pragma unroll
             for (int k = 0; k < 9; ++k) {

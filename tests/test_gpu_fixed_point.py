@@ -113,3 +113,90 @@ def test_time_factors(mu, dagger):
         mdwf.mdwf_set_chemical_potential(c.h, mu)
         emax, _ = rel_err(c.apply(odd, F64, dagger)[0], oracle.m(odd, U, p, dagger=dagger))
     assert emax <= 1e-12
+
+
+def far_apart(odd, k, part):
+    """odd with its colours, or its spins, 1, 2^-k and 2^-2k (a fourth spin: zero) in size."""
+    f = 2.0 ** (-k * np.arange(3.0))
+    return odd * f if part == "colours" else odd * np.append(f, 0.0)[:, None]
+
+
+def assert_each_part(got, ref, tol):
+    """Every (spin, colour) component within tol of its own largest element of the field."""
+    err = np.abs(got - ref).reshape(-1, 12).max(0)
+    top = np.abs(ref).reshape(-1, 12).max(0)
+    assert (err <= tol * top).all(), err / top
+
+
+# FP64 arithmetic: about 200 roundings a component and hop, 2e-14 at worst. Fixed point, where it is taken: 1.5 units of
+# the last place in the root mean square, six times that over the components of a field, against terms that add
+# up to 2^(54 - 7) units (a part 2^-7 of the largest component) times a link entry of 0.4: 1.6e-13 at the edge.
+PARTS_TOL = 2e-13
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("k", [1, 3, 6, 8, 20, 40])
+@pytest.mark.parametrize("shape", [0, 1])
+def test_colours_that_do_not_mix(shape, k, dagger):
+    """Links diagonal in colour (free fields, Abelian backgrounds) never add one colour to another in M, so a small
+    colour keeps its relative accuracy beside a large one."""
+    dims, Ls = [(DIMS, LS), ((8, 8, 4, 8), 10)][shape]
+    rng = np.random.default_rng(11)
+    ph = rng.uniform(-np.pi, np.pi, (*dims[::-1], 4, 2))
+    ph = np.concatenate([ph, -ph.sum(-1, keepdims=True)], -1)
+    U = np.exp(1j * ph)[..., None] * np.eye(3)
+    odd = far_apart(oracle.split(sy.gaussian_field(dims, Ls, 2411), dims)[1], k, "colours")
+    p = oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02)
+    ref = oracle.m(odd, U, p, dagger=dagger)
+    with Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.02, U) as c:
+        for sites in (0, 128 // Ls):
+            mdwf.mdwf_set_tuning(c.h, F64, 1, sites)
+            assert_each_part(c.apply(odd, F64, dagger)[0], ref, PARTS_TOL)
+
+
+@pytest.mark.parametrize("k", [6, 9, 20, 40])
+def test_one_colour_a_site(k):
+    """Each site holds one colour only, of a size of its own: the neighbours of a site differ in both."""
+    rng = np.random.default_rng(12)
+    U = np.broadcast_to(np.eye(3), (*DIMS[::-1], 4, 3, 3)).astype(complex)
+    odd = far_apart(oracle.split(sy.gaussian_field(DIMS, LS, 2412), DIMS)[1], k, "colours")
+    odd = odd * (rng.integers(0, 3, odd.shape[1])[:, None] == np.arange(3))[:, None, :]
+    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+        got = c.apply(odd, F64)[0]
+    assert_each_part(got, oracle.m(odd, U, oracle.Params(DIMS, LS, 1.8, 1.5, 0.5, 0.02)), PARTS_TOL)
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("k", [6, 9, 20, 40])
+def test_spins_that_do_not_mix(k, dagger):
+    """One hop adds to the upper spins only themselves and the lower ones: with the field on the even sites alone,
+    D_DW on the odd sites is one hop, and its small upper spins keep their accuracy."""
+    U = sy.gauge_field(DIMS, 0.7, 1413)
+    psi = sy.gaussian_field(DIMS, LS, 2413)
+    odd = oracle.split(psi, DIMS)[1]
+    psi = oracle.join(far_apart(oracle.split(psi, DIMS)[0], k, "spins"), 0 * odd, DIMS)
+    p = oracle.Params(DIMS, LS, 1.8, 1.5, 0.5, 0.02)
+    ref = oracle.ddw(psi, U, p, dagger=dagger)
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+        mdwf.mdwf_apply_full(c.h, out, torch.from_numpy(psi).cuda(), dagger=dagger)
+        torch.cuda.synchronize()
+    got, ref = (oracle.split(f, DIMS)[1] for f in (out.cpu().numpy(), ref))
+    assert_each_part(got, ref, PARTS_TOL)
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("k", [2, 6, 20, 40])
+def test_links_with_small_rows(k, dagger):
+    """Links that are not unitary, diagonal in colour with entries 1, 2^-k and 2^-2k."""
+    U = np.broadcast_to(np.diag(2.0 ** (-k * np.arange(3.0))), (*DIMS[::-1], 4, 3, 3)).astype(complex)
+    psi = sy.gaussian_field(DIMS, LS, 2414)
+    psi = oracle.join(oracle.split(psi, DIMS)[0], 0 * oracle.split(psi, DIMS)[1], DIMS)
+    p = oracle.Params(DIMS, LS, 1.8, 1.5, 0.5, 0.02)
+    ref = oracle.ddw(psi, U, p, dagger=dagger)
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+        mdwf.mdwf_apply_full(c.h, out, torch.from_numpy(psi).cuda(), dagger=dagger)
+        torch.cuda.synchronize()
+    got, ref = (oracle.split(f, DIMS)[1] for f in (out.cpu().numpy(), ref))
+    assert_each_part(got, ref, PARTS_TOL)
