@@ -83,51 +83,72 @@ __global__ void __launch_bounds__(128) layout_kernel(Field<P> even, Field<P> odd
     }
 }
 
-// fx, fx_exp: the fixed-point copy (fx.cuh), or null
-__global__ void gauge_pack_kernel(double2* u64, float* u32, int4* fx, int* fx_exp, const double2* __restrict__ U,
-                                  Geom g) {
-    const long long V = 2 * g.Vh;
-    const long long n = V * 4;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int mu = (int)(i % 4);
-        const long long lex = i / 4;
-        long long q = lex;
+// The user's links U[site][mu][9] to the FP64, FP32 and (unless fx is null) fixed-point copies, per parity and
+// direction. A block takes kPackSites consecutive sites; the two sites of a pair (2k, 2k + 1) differ in parity and have
+// the same index k in their copies, so of each parity and direction the block writes one contiguous run. Read and
+// written with consecutive 16-byte accesses, turned in shared memory. (A thread that walked its link's
+// 144 bytes in every copy took 212 us on 16^3 x 32, 140 without the fixed-point copy; now 58 us, 4.7 TB/s.)
+constexpr int kPackSites = 32, kPackLinks = 4 * kPackSites;
+__global__ void __launch_bounds__(kPackLinks) gauge_pack_kernel(double2* u64, float4* u32, int4* fx, int* fx_exp,
+                                                                const double* __restrict__ U, Geom g) {
+    __shared__ double2 tile[kPackLinks * 9];
+    __shared__ int swapped[kPackSites / 2];  // whether site 2k of the block is odd
+    __shared__ int exps[kPackLinks];
+    const long long base = (long long)blockIdx.x * kPackSites, left = 2 * g.Vh - base;
+    const int sites = left < kPackSites ? (int)left : kPackSites, links = 4 * sites, tid = threadIdx.x;
+    const double* src = U + base * 72;
+    const bool wide = (reinterpret_cast<size_t>(U) & 15) == 0;  // a caller's doubles need not be 16-byte aligned
+    for (int i = tid; i < links * 9; i += kPackLinks)
+        tile[i] = wide ? __ldg(reinterpret_cast<const double2*>(src) + i)
+                       : make_double2(__ldg(src + 2 * i), __ldg(src + 2 * i + 1));
+    if (tid < sites / 2) {
+        long long q = base + 2 * tid;
         const int x = (int)(q % g.X); q /= g.X;
         const int y = (int)(q % g.Y); q /= g.Y;
         const int z = (int)(q % g.Z); q /= g.Z;
-        const int t = (int)q;
-        const int par = (x + y + z + t) & 1;
-        const long long l = ((long long)par * 4 + mu) * g.Vh + (lex >> 1);
-        const double2* src = U + i * 9;
+        swapped[tid] = (x + y + z + (int)q) & 1;
+    }
+    __syncthreads();
+    // link r of the block in the order of the copies, r = (parity 4 + mu) sites / 2 + k: its place in the tile and there
+    const int half = sites / 2;
+    auto place = [&](int r) {
+        const int q = r / half, k = r % half;
+        return (2 * k + ((q >> 2) ^ swapped[k])) * 4 + (q & 3);
+    };
+    auto index = [&](int r) { return (long long)(r / half) * g.Vh + base / 2 + r % half; };
+    if (fx && tid < links) {
+        double v[18];
+        const double2* u = tile + place(tid) * 9;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            double2 d = src[k];
-            u64[l * 9 + k] = d;
-            u32[l * 20 + 2 * k] = (float)d.x;
-            u32[l * 20 + 2 * k + 1] = (float)d.y;
+            v[2 * k] = u[k].x;
+            v[2 * k + 1] = u[k].y;
         }
-        u32[l * 20 + 18] = 0.f;
-        u32[l * 20 + 19] = 0.f;
+        int e = fx_exponent<18>(v);
+        if (e != kFxZero && !fx_link_even(v)) e = kFxRaw;  // such a link is read from the FP64 copy
+        exps[tid] = e;
+        fx_exp[index(tid)] = e;
+    }
+    __syncthreads();
+    for (int i = tid; i < links * 9; i += kPackLinks) {
+        const int r = i / 9, w = i % 9;
+        const double2 d = tile[place(r) * 9 + w];
+        const long long at = index(r) * 9 + w;
+        u64[at] = d;
         if (fx) {
-            double v[18];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                v[2 * k] = src[k].x;
-                v[2 * k + 1] = src[k].y;
+            int4 o = make_int4(0, 0, 0, 0);
+            if (exps[r] != kFxRaw) {
+                fx_split(fx_mantissa<8>(d.x, exps[r]), o.y, o.x);
+                fx_split(fx_mantissa<8>(d.y, exps[r]), o.w, o.z);
             }
-            int e = fx_exponent<18>(v);
-            if (e != kFxZero && !fx_link_even(v)) e = kFxRaw;
-            fx_exp[l] = e;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                int4 o = make_int4(0, 0, 0, 0);
-                if (e != kFxRaw) {  // such a link is read from the FP64 copy
-                    fx_split(fx_mantissa<8>(v[2 * k], e), o.y, o.x);
-                    fx_split(fx_mantissa<8>(v[2 * k + 1], e), o.w, o.z);
-                }
-                fx[l * 9 + k] = o;
-            }
+            fx[at] = o;
         }
+    }
+    for (int i = tid; i < links * 5; i += kPackLinks) {  // 18 floats and two zeros
+        const int r = i / 5, w = i % 5;
+        const double2* u = tile + place(r) * 9 + 2 * w;
+        const double2 a = u[0], b = w < 4 ? u[1] : make_double2(0.0, 0.0);
+        u32[index(r) * 5 + w] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
     }
 }
 
@@ -220,9 +241,8 @@ int launch_join_full(mdwf_ctx* c, double* full, const void* even, const void* od
 int launch_gauge_pack(mdwf_ctx* c, const double* U) {
     const long long n = 2 * c->g.Vh * 4;
     LaunchScope scope(c, KB_LAYOUT * 3 + MDWF_F64, n * (144.0 * (c->gauge_fx ? 3 : 2) + 80.0), 0.0);
-    gauge_pack_kernel<<<grid_for(n, 256), 256, 0, c->stream>>>((double2*)c->gauge[0], (float*)c->gauge[1],
-                                                                (int4*)c->gauge_fx, c->gauge_fx_exp,
-                                                                (const double2*)U, c->g);
+    gauge_pack_kernel<<<(unsigned)((2 * c->g.Vh + kPackSites - 1) / kPackSites), kPackLinks, 0, c->stream>>>(
+        (double2*)c->gauge[0], (float4*)c->gauge[1], (int4*)c->gauge_fx, c->gauge_fx_exp, U, c->g);
     return check_launch();
 }
 

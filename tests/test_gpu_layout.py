@@ -7,9 +7,10 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
+import oracle
 import paper_1206_5214_gb300 as mdwf
 import synthetic as sy
-from _gpu import Ctx
+from _gpu import Ctx, rel_err
 
 pytestmark = pytest.mark.gpu
 F64, F32, F16N = mdwf.MDWF_F64, mdwf.MDWF_F32, mdwf.MDWF_F16N
@@ -59,3 +60,19 @@ def test_full_fields_unaligned(dims, Ls):
             torch.cuda.synchronize()
             outs.append(out)
         assert torch.equal(*outs)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 2, 2, 6), (6, 4, 2, 4), (4, 2, 6, 10)])
+def test_links(dims, offset):
+    """Links loaded from aligned and unaligned buffers, with whole and partial blocks of sites: M in every precision
+    against the oracle (each precision reads a copy of its own)."""
+    U = sy.gauge_field(dims, 0.5, 1502)
+    buf = doubles(U.size * 2, offset)
+    buf.copy_(torch.from_numpy(U.reshape(-1).view(np.float64)))
+    odd = oracle.split(sy.gaussian_field(dims, 4, 2502), dims)[1]
+    ref = oracle.m(odd, U, oracle.Params(dims, 4, 1.8, 1.5, 0.5, 0.02))
+    with Ctx(dims, 4, 1.8, 1.5, 0.5, 0.02, sy.unit_gauge(dims)) as c:
+        mdwf.mdwf_load_gauge(c.h, buf)
+        for prec, tol in ((F64, 1e-12), (F32, 1e-5), (F16N, 1e-2)):
+            assert rel_err(c.apply(odd, prec)[0], ref)[0] <= tol
