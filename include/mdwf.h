@@ -200,10 +200,12 @@ int mdwf_get_s_coefficients(const mdwf_ctx *ctx, double *b5s, double *c5s, int *
  * Loads the SU(3) links U_mu(x) (Eq. D^Wilson) from complex128
  * U[t][z][y][x][mu][3][3] in host (where = MDWF_HOST) or device memory.
  * The data is copied into per-parity, per-direction link arrays in FP64 and
- * FP32 (the FP32 copy also serves the FP16+norm operator), and for the FP64
- * hops in 64-bit fixed point (not on t-slabs); the caller's buffer
- * may be reused once the call returns (host) or once the stream has passed
- * this point (device).
+ * FP32 (the FP32 copy also serves the FP16+norm operator), 228 B a link, and
+ * for the FP64 hops in 64-bit fixed point, 144 B more (not on t-slabs, nor on a
+ * device that would have no room for four FP64 fields beside it: FP64 hops then
+ * run in FP64 arithmetic, 3.4 times slower). The caller's buffer may be reused
+ * once the call returns (host) or once the stream has passed this point
+ * (device).
  */
 int mdwf_load_gauge(mdwf_ctx *ctx, const double *U, int where);
 

@@ -633,20 +633,32 @@ int mdwf_load_gauge(mdwf_ctx* c, const double* U, int where) {
     if ((st = cuda_status(cudaSetDevice(c->device)))) return st;
     const size_t nlink = (size_t)c->g.Vh * 2 * 4;
     if (!c->gauge[0]) {
-        // the FP64 and FP32 copies and, not on t-slabs, the fixed-point copy that the FP64 hops read: one allocation
-        // (each takes a quarter of a millisecond, beside 2 ms for a context)
+        // the FP64 and FP32 copies and the fixed-point copy that the FP64 hops read: one allocation (each takes a
+        // quarter of a millisecond, beside 2 ms for a context). T-slabs have no third copy. Where it would take the
+        // room that the rest of an application needs (four FP64 fields), only its exponents are there, all raw: the FP64
+        // hops then run in FP64 arithmetic.
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t b64 = up(nlink * link_store_bytes(MDWF_F64)), b32 = up(nlink * link_store_bytes(MDWF_F32));
-        const size_t bfx = c->slab ? 0 : nlink * (144 + sizeof(int));
-        void* base = nullptr;
-        if ((st = cuda_status(cudaMalloc(&base, b64 + b32 + bfx)))) return st;
-        c->gauge[0] = base;
-        c->gauge[1] = (char*)base + b64;
-        if (!c->slab) {
-            c->gauge_fx = (char*)base + b64 + b32;
-            c->gauge_fx_exp = (int*)((char*)c->gauge_fx + nlink * 144);
+        const size_t bexp = c->slab ? 0 : up(nlink * sizeof(int));
+        size_t bfx = c->slab ? 0 : nlink * 144, free_b = 0, total_b = 0;
+        const size_t need = b64 + b32 + bexp + bfx + 4 * field_bytes(MDWF_F64, c->g, 1);
+        if (need > ((size_t)512 << 20)) {  // a lattice that can be short of room (the question costs 0.4 ms)
+            if ((st = cuda_status(cudaMemGetInfo(&free_b, &total_b)))) return st;
+            if (free_b < need) bfx = 0;
         }
-        if ((st = canary_fill(base, b64 + b32 + bfx))) return st;
+        char* base = nullptr;
+        st = cuda_status(cudaMalloc(&base, b64 + b32 + bexp + bfx));
+        if (st == MDWF_ENOMEM && bfx) {
+            cudaGetLastError();
+            bfx = 0;
+            st = cuda_status(cudaMalloc(&base, b64 + b32 + bexp));
+        }
+        if (st) return st;
+        c->gauge[0] = base;
+        c->gauge[1] = base + b64;
+        if (!c->slab) c->gauge_fx_exp = (int*)(base + b64 + b32);
+        if (bfx) c->gauge_fx = base + b64 + b32 + bexp;
+        if ((st = canary_fill(base, b64 + b32 + bexp + bfx))) return st;
     }
     const double* src = U;
     void* stage = nullptr;

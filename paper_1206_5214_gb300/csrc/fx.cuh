@@ -184,7 +184,8 @@ __device__ __forceinline__ void fx_store(const Field<MDWF_F64>& f, int* e, long 
     e[sr * f.Ls + s] = x;
 }
 
-// Fixed-point links: [link][9] of (re lo, re hi, im lo, im hi), and one exponent per link.
+// Fixed-point links: [link][9] of (re lo, re hi, im lo, im hi), and one exponent per link. A context without
+// them has the exponents alone, all kFxRaw.
 struct FxGauge {
     const int4* u;
     const int* e;

@@ -83,11 +83,12 @@ __global__ void __launch_bounds__(128) layout_kernel(Field<P> even, Field<P> odd
     }
 }
 
-// The user's links U[site][mu][9] to the FP64, FP32 and (unless fx is null) fixed-point copies, per parity and
-// direction. A block takes kPackSites consecutive sites; the two sites of a pair (2k, 2k + 1) differ in parity and have
-// the same index k in their copies, so of each parity and direction the block writes one contiguous run. Read and
-// written with consecutive 16-byte accesses, turned in shared memory. (A thread that walked its link's
-// 144 bytes in every copy took 212 us on 16^3 x 32, 140 without the fixed-point copy; now 58 us, 4.7 TB/s.)
+// The user's links U[site][mu][9] to the FP64, FP32 and fixed-point copies, per parity and direction (no fixed-point
+// copy: fx is null; fx_exp, unless null too, then marks every link as raw). A block takes kPackSites consecutive
+// sites; the two sites of a pair (2k, 2k + 1) differ in parity and have the same index k in their copies, so of each
+// parity and direction the block writes one contiguous run. Read and written with consecutive 16-byte accesses,
+// turned in shared memory. (A thread that walked its link's 144 bytes in every copy took 202 us on 16^3 x 32, 134
+// without the fixed-point copy; now 58 us, 4.7 TB/s.)
 constexpr int kPackSites = 32, kPackLinks = 4 * kPackSites;
 __global__ void __launch_bounds__(kPackLinks) gauge_pack_kernel(double2* u64, float4* u32, int4* fx, int* fx_exp,
                                                                 const double* __restrict__ U, Geom g) {
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(kPackLinks) gauge_pack_kernel(double2* u64, fl
         return (2 * k + ((q >> 2) ^ swapped[k])) * 4 + (q & 3);
     };
     auto index = [&](int r) { return (long long)(r / half) * g.Vh + base / 2 + r % half; };
+    if (!fx && fx_exp && tid < links) fx_exp[index(tid)] = kFxRaw;
     if (fx && tid < links) {
         double v[18];
         const double2* u = tile + place(tid) * 9;

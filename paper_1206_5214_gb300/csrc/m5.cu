@@ -64,10 +64,15 @@ __global__ void __launch_bounds__(256, P == MDWF_F64 ? 1 : 4) m5_kernel(Field<P>
             R h0[12], h1[12];
             in.load_half(sr, sw ? up : dn, 0, h0);
             in.load_half(sr, sw ? dn : up, 1, h1);
+            // FP64: no product with w0 = 1 (2 FP64 operations a clock and SM); the others: no second branch (registers)
+            if (P != MDWF_F64 || w0 != R(1)) {
+#pragma unroll
+                for (int k = 0; k < 24; ++k) v[k] *= w0;
+            }
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
-                v[k] = fma(f0, h0[k], w0 * v[k]);
-                v[12 + k] = fma(f1, h1[k], w0 * v[12 + k]);
+                v[k] = fma(f0, h0[k], v[k]);
+                v[12 + k] = fma(f1, h1[k], v[12 + k]);
             }
         }
         if (XPAY) {

@@ -790,7 +790,7 @@ struct mdwf_ctx {
     bool have_gauge = false;
     void* gauge[2] = {nullptr, nullptr};  // FP64 and FP32 copies, in one allocation with
     void* gauge_fx = nullptr;             // the fixed-point copy (fx.cuh), 144 B per link as the FP64 one,
-    int* gauge_fx_exp = nullptr;          // and its exponents
+    int* gauge_fx_exp = nullptr;          // and its exponents (t-slabs: neither; short memory: exponents only)
     // Ls x Ls tables for the current mass list, FP64 and FP32, plus per-rhs masses
     double* tab64 = nullptr;
     float* tab32 = nullptr;

@@ -200,3 +200,42 @@ def test_links_with_small_rows(k, dagger):
         torch.cuda.synchronize()
     got, ref = (oracle.split(f, DIMS)[1] for f in (out.cpu().numpy(), ref))
     assert_each_part(got, ref, PARTS_TOL)
+
+
+def test_links_without_a_fixed_point_copy():
+    """With little device memory free the links are held without the fixed-point copy (228 instead of 372 B each),
+    and the FP64 operator runs in FP64 arithmetic."""
+    dims, Ls, nlink = (16, 16, 16, 16), 32, 4 * 16 ** 4
+    field = dims[0] ** 4 // 2 * Ls * 192
+    U = sy.gauge_field(dims, 0.3, 1415)
+    odd = oracle.split(sy.gaussian_field(dims, Ls, 2415), dims)[1]
+    outs, taken = [], []
+    for short in (False, True):
+        torch.cuda.empty_cache()
+        with Ctx((4, 4, 2, 2), 4, 1.8, 1.5, 0.5, 0.02, sy.unit_gauge((4, 4, 2, 2))) as c:  # loads the kernels
+            c.apply(np.zeros((4, 32, 4, 3), complex), F64)
+        Ud = torch.from_numpy(U).cuda()
+        h = mdwf.mdwf_create(dims, Ls, 1.8, 1.5, 0.5, 0.02)
+        try:
+            src, dst = (torch.empty(field, dtype=torch.uint8, device="cuda") for _ in range(2))
+            mdwf.mdwf_field_import(h, src, torch.from_numpy(odd).cuda(), F64, 1)
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            free = torch.cuda.mem_get_info()[0]
+            filler = torch.empty(free - 7 * field // 2, dtype=torch.uint8, device="cuda") if short else None
+            free = torch.cuda.mem_get_info()[0]
+            mdwf.mdwf_load_gauge(h, Ud)
+            taken.append(free - torch.cuda.mem_get_info()[0])
+            mdwf.mdwf_apply(h, dst, src, F64, 1)
+            torch.cuda.synchronize()
+            del filler
+            torch.cuda.empty_cache()
+            out = torch.empty((1, Ls, 8 * 16 ** 3, 4, 3), dtype=torch.complex128, device="cuda")
+            mdwf.mdwf_field_export(h, out, dst, F64, 1)
+            outs.append(out.cpu().numpy()[0])
+        finally:
+            mdwf.mdwf_destroy(h)
+    page = 4 << 20   # the driver's granularity
+    assert taken[0] > 372 * nlink - page and taken[1] < 228 * nlink + page, taken
+    ref = oracle.m(odd, U, oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02))
+    assert all(rel_err(o, ref)[0] <= 1e-12 for o in outs)
