@@ -229,9 +229,9 @@ int mdwf_field_export(mdwf_ctx *ctx, double *dst, const void *src, int prec, int
  * mf_per_rhs: NULL (every right-hand side uses the context's mf) or nrhs
  * masses (host memory), one per right-hand side.
  * FP64 hopping sums run on 64-bit integers with one exponent per (site, s)
- * spinor where its spins and colours are within 2^7 of each other, and in FP64
- * arithmetic elsewhere: every component keeps FP64's accuracy, at worst 2^-41
- * of the terms it is made of.
+ * spinor where its spins and colours are within 2^8 of each other, and in FP64
+ * arithmetic elsewhere: every component keeps FP64's accuracy, at the edge of
+ * that rule 7e-13 of the terms it is made of.
  */
 int mdwf_apply(mdwf_ctx *ctx, void *out, const void *in, int prec, int nrhs, const double *mf_per_rhs);
 

@@ -126,8 +126,7 @@ __global__ void __launch_bounds__(kPackLinks) gauge_pack_kernel(double2* u64, fl
             v[2 * k] = u[k].x;
             v[2 * k + 1] = u[k].y;
         }
-        int e = fx_exponent<18>(v);
-        if (e != kFxZero && !fx_link_even(v)) e = kFxRaw;  // such a link is read from the FP64 copy
+        const int e = fx_link_exponent(v);  // kFxRaw: the link is read from the FP64 copy
         exps[tid] = e;
         fx_exp[index(tid)] = e;
     }

@@ -130,12 +130,12 @@ def assert_each_part(got, ref, tol):
 
 # FP64 arithmetic: about 200 roundings a component and hop, 2e-14 at worst. Fixed point, where it is taken: 1.5 units of
 # the last place in the root mean square, six times that over the components of a field, against terms that add
-# up to 2^(54 - 7) units (a part 2^-7 of the largest component) times a link entry of 0.4: 1.6e-13 at the edge.
-PARTS_TOL = 2e-13
+# up to 2^(54 - 8) units (a part 2^-8 of the largest component) times a link entry of 0.57: 2.3e-13 at the edge.
+PARTS_TOL = 3e-13
 
 
 @pytest.mark.parametrize("dagger", [False, True])
-@pytest.mark.parametrize("k", [1, 3, 6, 8, 20, 40])
+@pytest.mark.parametrize("k", [1, 4, 7, 9, 20, 40])
 @pytest.mark.parametrize("shape", [0, 1])
 def test_colours_that_do_not_mix(shape, k, dagger):
     """Links diagonal in colour (free fields, Abelian backgrounds) never add one colour to another in M, so a small
@@ -154,7 +154,7 @@ def test_colours_that_do_not_mix(shape, k, dagger):
             assert_each_part(c.apply(odd, F64, dagger)[0], ref, PARTS_TOL)
 
 
-@pytest.mark.parametrize("k", [6, 9, 20, 40])
+@pytest.mark.parametrize("k", [7, 9, 20, 40])
 def test_one_colour_a_site(k):
     """Each site holds one colour only, of a size of its own: the neighbours of a site differ in both."""
     rng = np.random.default_rng(12)
@@ -167,7 +167,7 @@ def test_one_colour_a_site(k):
 
 
 @pytest.mark.parametrize("dagger", [False, True])
-@pytest.mark.parametrize("k", [6, 9, 20, 40])
+@pytest.mark.parametrize("k", [7, 9, 20, 40])
 def test_spins_that_do_not_mix(k, dagger):
     """One hop adds to the upper spins only themselves and the lower ones: with the field on the even sites alone,
     D_DW on the odd sites is one hop, and its small upper spins keep their accuracy."""
@@ -186,7 +186,7 @@ def test_spins_that_do_not_mix(k, dagger):
 
 
 @pytest.mark.parametrize("dagger", [False, True])
-@pytest.mark.parametrize("k", [2, 6, 20, 40])
+@pytest.mark.parametrize("k", [2, 7, 20, 40])
 def test_links_with_small_rows(k, dagger):
     """Links that are not unitary, diagonal in colour with entries 1, 2^-k and 2^-2k."""
     U = np.broadcast_to(np.diag(2.0 ** (-k * np.arange(3.0))), (*DIMS[::-1], 4, 3, 3)).astype(complex)
