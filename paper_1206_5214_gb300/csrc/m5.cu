@@ -20,18 +20,21 @@ __device__ __forceinline__ void store_m5(const Field<P>& f, int* exp, long long 
     f.store(sr, s, v);
 }
 
-// FP32 and FP16+norm: four blocks per SM (64 registers). At 75 registers and three blocks M_phi of 16^3 x 32 x 16 took
-// 26.6 us in FP16+norm and 31.0 in FP32, now 24.5 and 30.0; A^dag 34.8 and 38.8, now 32.7 and 36.6.
-template <int P, bool XPAY>
-__global__ void __launch_bounds__(256, P == MDWF_F64 ? 1 : 4) m5_kernel(Field<P> out, Field<P> in, Field<P> xf,
-                                                 const typename PrecTraits<P>::real* tab,
-                                                 const typename PrecTraits<P>::real* mass,
-                                                 typename PrecTraits<P>::real coef, Geom g, int sop, int swap,
-                                                 SCoef<typename PrecTraits<P>::real> sc, const double* mask, int* out_exp) {
+// FORM: the operators that read a spinor and its two neighbours straight from memory (below), whole columns in
+// shared memory, or dense tables. Blocks per SM: FP32 and FP16+norm eight (64 registers; at 75 and six blocks M_phi
+// of 16^3 x 32 x 16 took 31.0 and 26.6 us, now 29.8 and 24.6). FP64 direct four, 71 us (six: 105); FP64 columns,
+// which wait for the FP64 pipe and for each other, six: A^dag 144 us at 80 registers with some spilled, 152 with
+// five, 176 with four, and 162 with four and no rule on the parts of a spinor (fx.cuh); FP64 dense four.
+enum { M5_DIRECT, M5_COLUMNS, M5_DENSE };
+template <int P, bool XPAY, int FORM>
+__global__ void __launch_bounds__(128, P != MDWF_F64 ? 8 : FORM == M5_COLUMNS ? 6 : 4)
+    m5_kernel(Field<P> out, Field<P> in, Field<P> xf, const typename PrecTraits<P>::real* tab,
+              const typename PrecTraits<P>::real* mass, typename PrecTraits<P>::real coef, Geom g, int sop, int swap,
+              SCoef<typename PrecTraits<P>::real> sc, const double* mask, int* out_exp) {
     typedef typename PrecTraits<P>::real R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ls = g.Ls;
-    const bool dense = sop == SOP_DENSE;
+    constexpr bool dense = FORM == M5_DENSE;
     R* mat = reinterpret_cast<R*>(smem_raw);
     R* cs = mat + (dense ? 2 * Ls * Ls : 0);
     const int nrhs = (int)(gridDim.x / ((g.Vh + blockDim.y - 1) / blockDim.y));
@@ -46,14 +49,13 @@ __global__ void __launch_bounds__(256, P == MDWF_F64 ? 1 : 4) m5_kernel(Field<P>
     // since a neighbour's element may be overwritten). Chirality 0 (reals 0..11)
     // couples to s - 1 and chirality 1 to s + 1; the adjoint (swap) exchanges them;
     // the wrap-around term carries -m. Block-uniform.
-    const bool bidiag = sop == SOP_MPHI || sop == SOP_C || sop == SOP_MEE;
-    if (!dense && (sop == SOP_ID || (bidiag && (const void*)out.v != (const void*)in.v))) {
+    if constexpr (FORM == M5_DIRECT) {
         const long long site = sblk * blockDim.y + ly;
         if (site >= g.Vh) return;
         const long long sr = (long long)rhs * g.Vh + site;
         R v[24];
         in.load(sr, s, v);
-        if (bidiag) {
+        if (sop != SOP_ID) {
             R w0, w1;
             bidiag_weights(sop, sc, w0, w1);
             const R m = mass[rhs];
@@ -119,7 +121,7 @@ __global__ void __launch_bounds__(256, P == MDWF_F64 ? 1 : 4) m5_kernel(Field<P>
             for (int k = 12; k < 24; ++k) res[k] += mm * h[k];
         }
     } else {
-        // the shared-memory walk: register-held columns measured slower in this 256-thread kernel
+        // the shared-memory walk: register-held columns measured slower in this kernel
         const SMass<R> sm{mass[rhs], mass[kMaxRhs + rhs]};
         block_columns(cs, blockDim.y, Ls, sop, swap != 0, sc, sm, tid, nthr, false);
         __syncthreads();
@@ -158,17 +160,17 @@ static int launch_m5_t(mdwf_ctx* c, const M5Launch& m) {
     const double n5 = (double)g.Vh * g.Ls * m.nrhs;
     LaunchScope scope(c, (m.x ? KB_M5_XPAY : KB_M5) * 3 + P, n5 * site_bytes(P) * (m.x ? 3.0 : 2.0),
                       n5 * (144.0 + (m.x ? 24.0 : 0.0)));
-    if (m.x) {
-        auto k = m5_kernel<P, true>;
+    auto launch = [&](auto k) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, coef, g, m.sop, m.swap, sc, m.mask,
-                                          m.out_exp);
-    } else {
-        auto k = m5_kernel<P, false>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, coef, g, m.sop, m.swap, sc, m.mask,
-                                          m.out_exp);
-    }
+        k<<<grid, block, smem, c->stream>>>(out, in, xf, tab, mass, coef, g, m.sop, m.swap, sc, m.mask, m.out_exp);
+    };
+    const bool bidiag = m.sop == SOP_MPHI || m.sop == SOP_C || m.sop == SOP_MEE;
+    if (m.sop == SOP_DENSE)
+        m.x ? launch(m5_kernel<P, true, M5_DENSE>) : launch(m5_kernel<P, false, M5_DENSE>);
+    else if (m.sop == SOP_ID || (bidiag && m.out != m.in))
+        m.x ? launch(m5_kernel<P, true, M5_DIRECT>) : launch(m5_kernel<P, false, M5_DIRECT>);
+    else
+        m.x ? launch(m5_kernel<P, true, M5_COLUMNS>) : launch(m5_kernel<P, false, M5_COLUMNS>);
     return check_launch();
 }
 
