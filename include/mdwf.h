@@ -426,8 +426,12 @@ int mdwf_counters(const mdwf_ctx *ctx, long long *launches, long long applies[3]
  * M^dag application of the context's own scratch fields, and the fastest is
  * kept for later launches of that (prec, nrhs). Allocates scratch fields and
  * synchronises the stream. *sites_per_block receives the choice (may be NULL).
- * mdwf_set_tuning / mdwf_get_tuning store and read a choice directly, so a
- * caller can keep tuned values across runs (0 = the default shape).
+ * mdwf_set_tuning stores a choice directly, so a caller can keep tuned values
+ * across runs (0 = the default shape); mdwf_get_tuning reads the sites per
+ * block in use. On the smallest lattices the default shape of the FP32 and FP64
+ * operators gives a column to four or two threads, with a fourth or half of
+ * the sites per block: it is a candidate, and storing its number of sites
+ * selects it.
  */
 int mdwf_autotune(mdwf_ctx *ctx, int prec, int nrhs, int *sites_per_block);
 int mdwf_set_tuning(mdwf_ctx *ctx, int prec, int nrhs, int sites_per_block);

@@ -364,8 +364,9 @@ int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int 
 }
 
 // Times M + M^dag for every candidate block shape on scratch fields and keeps
-// the fastest for (prec, nrhs). Candidates: whole s-columns per block with
-// 32, 64 or 128 threads at most (the hop kernels are built for 128).
+// the fastest for (prec, nrhs). Candidates: the whole s-columns of 32, 64 or 128
+// threads (the hop kernels are built for 128), among them the one that hop_shape
+// takes as the split form.
 int tune_hop(mdwf_ctx* c, int prec, int nrhs, int* chosen) {
     const size_t fb = field_bytes(prec, c->g, nrhs);
     int st;
@@ -475,7 +476,8 @@ static int create_context(mdwf_ctx** out, const int dims[4], int Ls, double M5, 
     c->autotune = opts && opts->autotune;
     c->slab = slab;
     // the default mass tables, so that an apply needs no host round trip
-    if ((st = ensure_tables(c, 1, nullptr)) ||
+    if ((st = cuda_status(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev))) ||
+        (st = ensure_tables(c, 1, nullptr)) ||
         (st = cuda_status(cudaMalloc(&c->nbr, sizeof(int) * 16 * (size_t)c->g.Vh))) ||
         (st = cuda_status(cudaMalloc(&c->dev_err, sizeof(int)))) ||
         (st = cuda_status(cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream))) ||
@@ -799,7 +801,7 @@ int mdwf_set_tuning(mdwf_ctx* c, int prec, int nrhs, int sites_per_block) {
 
 int mdwf_get_tuning(const mdwf_ctx* c, int prec, int nrhs, int* sites_per_block) {
     if (!c || !valid_prec(prec) || nrhs < 1 || nrhs > 64 || !sites_per_block) return MDWF_EINVAL;
-    *sites_per_block = hop_sites_per_block(c, prec, nrhs);
+    *sites_per_block = hop_shape(c, prec, nrhs).sites;
     return MDWF_OK;
 }
 

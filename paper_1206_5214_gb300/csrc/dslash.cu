@@ -9,33 +9,26 @@ namespace mdwf {
 
 template <int P> int launch_hop_t(mdwf_ctx* c, const HopLaunch& h);
 
-// 4d sites per block: the autotuned value for (precision, nrhs) if there is
-// one, else as many whole s-columns as fit 128 threads.
-int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs) {
-    const int t = (nrhs >= 1 && nrhs <= 64) ? c->sb_tune[prec][nrhs] : 0;
-    if (t > 0) return t;
-    const int sb = 128 / c->g.Ls;
-    return sb < 1 ? 1 : sb;
-}
-
-// The block shape of a hop launch. Where the whole s-columns of 128 threads make so few blocks that the time of a
-// hop is that of one thread's chain of eight neighbours, four or (FP64) two threads share a column (STAGE 5 and 6 of the
-// kernel). M alone in us, one, two and four threads a column, by the number of ordinary blocks:
+// The block shape of a hop launch: as many whole s-columns as fit 128 threads, or the autotuned number. Where such blocks
+// are so few that the time of a hop is that of one thread's chain of eight neighbours, four or (FP64) two threads share a
+// column (STAGE 5 and 6 of the kernel) and a block holds a fourth or half of the columns. M alone in us, one, two and four
+// threads a column, by the number of ordinary blocks on 152 SMs:
 //   FP32: 8 blocks 16.4, -, 13.7; 128 blocks 17.0, -, 14.4; 140 blocks 20.5, -, 16.5; 256 blocks 16.5, -, 20.5
 //   FP64: 8 blocks 47, 34, 30; 64 blocks 49, 34, 34; 128 blocks 49, 43, 56; 205 blocks 64, 46, 72; 256 blocks 64, 77, 95
 // FP32 gains while the ordinary form leaves an SM at most one block. The FP64 split forms run three blocks per SM:
 // two threads a column pay while those blocks are one wave (205 blocks make 410, 256 make 512, of 456), four while
 // the integer pipe is not the limit.
-// Not for FP16+norm (its sums would round differently), a tuned block shape or a chosen load strategy.
-constexpr int kSplit4BlocksF32 = 152, kSplit4BlocksF64 = 64, kSplit2BlocksF64 = 3 * 152 / 2;
+// Not for FP16+norm (its sums would round differently) or a chosen load strategy. A tuned number of sites that is the
+// split form's selects that form (so the tuner, whose candidates hold it, can choose it); any other the ordinary one.
 HopShape hop_shape(const mdwf_ctx* c, int prec, int nrhs) {
-    const int sb = hop_sites_per_block(c, prec, nrhs);
-    const long long blocks = (c->g.Vh + sb - 1) / sb * nrhs;
-    const bool tuned = nrhs >= 1 && nrhs <= 64 && c->sb_tune[prec][nrhs] > 0;
-    if (prec == MDWF_F16N || c->slab || tuned || c->hop_stage[prec] != 0) return {sb, 1};
-    if (blocks <= (prec == MDWF_F64 ? kSplit4BlocksF64 : kSplit4BlocksF32)) return {32 / c->g.Ls, 4};
-    if (prec == MDWF_F64 && blocks <= kSplit2BlocksF64) return {64 / c->g.Ls, 2};
-    return {sb, 1};
+    const int full = 128 / c->g.Ls, tuned = nrhs >= 1 && nrhs <= 64 ? c->sb_tune[prec][nrhs] : 0;
+    const long long blocks = (c->g.Vh + full - 1) / full * nrhs;
+    int split = 1;
+    if (prec == MDWF_F32 && blocks <= c->sms) split = 4;
+    if (prec == MDWF_F64) split = blocks * 152 <= c->sms * 64 ? 4 : blocks * 2 <= c->sms * 3 ? 2 : 1;
+    if (c->slab || c->hop_stage[prec] != 0) split = 1;
+    const int sites = 128 / split / c->g.Ls;
+    return tuned > 0 && tuned != sites ? HopShape{tuned, 1} : HopShape{sites, split};
 }
 
 // The fused iteration drops its t field when the FUSE_R epilogue can rebuild

@@ -786,6 +786,7 @@ struct mdwf_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     mdwf::Geom g{};
+    int sms = 0;  // the device's multiprocessors
     double M5 = 0, b5 = 0, c5 = 0, mf = 0;
     bool have_gauge = false;
     void* gauge[2] = {nullptr, nullptr};  // FP64 and FP32 copies, in one allocation with
@@ -986,7 +987,6 @@ struct HopLaunch {
 int launch_hop(mdwf_ctx* c, int prec, const HopLaunch& h);
 // whether the fused CG iteration can run without its t field (HopLaunch::no_t)
 bool hop_no_t_ok(const mdwf_ctx* c, int prec, int nrhs);
-int hop_sites_per_block(const mdwf_ctx* c, int prec, int nrhs);
 // the 4d sites per block of a hop launch, and how many threads share each of its columns
 struct HopShape {
     int sites, split;
