@@ -37,44 +37,55 @@ def check(prec, got, ref):
     emax, el2 = rel_err(got, ref)
     assert (el2 <= 3e-3) if prec == F16N else (emax <= (1e-12 if prec == F64 else 1e-5)), (prec, emax, el2)
 
-# operator and adjoint, three precisions, a ragged lattice and Ls = 16
-for dims, Ls in (((4, 4, 4, 4), 8), ((2, 4, 6, 4), 6), ((4, 2, 2, 4), 16)):
+# operator and adjoint, three precisions, a ragged lattice and Ls = 16, each in the form with several threads a
+# column that these lattices get (the last one two in FP64) and in the ordinary form
+for dims, Ls in (((4, 4, 4, 4), 8), ((2, 4, 6, 4), 6), ((4, 2, 2, 4), 16), ((8, 8, 4, 8), 10)):
     U = sy.gauge_field(dims, 0.3, 1301)
     odd = oracle.split(sy.gaussian_field(dims, Ls, 2301), dims)[1]
     p = oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02)
     with Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.02, U) as c:
-        for prec in (F64, F32, F16N):
-            for dag in (False, True):
-                check(prec, c.apply(odd, prec, dag)[0], oracle.m(odd, U, p, dagger=dag))
+        for dag in (False, True):
+            ref = oracle.m(odd, U, p, dagger=dag)
+            for prec in (F64, F32, F16N):
+                for sites in (0, 128 // Ls):
+                    mdwf.mdwf_set_tuning(c.h, prec, 1, sites)
+                    check(prec, c.apply(odd, prec, dag)[0], ref)
+        mdwf.mdwf_set_tuning(c.h, F32, 1, 0)
         fin = c.upload(odd, F32)
         got = c.alloc(F32)
         mdwf.mdwf_apply_noalloc(c.h, got, fin, F32, 1, [0.02])
         torch.cuda.synchronize()
         check(F32, c.download(got, F32)[0], oracle.m(odd, U, p))
 
-# mixed solves: Ls = 16 (no t field) and Ls = 8, two right-hand sides
-for Ls in (16, 8):
+# mixed solves: Ls = 16 (no t field) and Ls = 8, two right-hand sides, and the FP64 solve, in both forms
+for Ls, tuned in ((16, False), (8, False), (16, True), (8, True)):
     dims = (4, 4, 4, 4)
     U = sy.gauge_field(dims, 0.3, 1302)
     b = sy.gaussian_field(dims, Ls, 2302, nrhs=2)
     h = mdwf.mdwf_create(dims, Ls, 1.8, 1.5, 0.5, 0.01)
+    xs = {}
     try:
         mdwf.mdwf_load_gauge(h, torch.from_numpy(U).cuda())
+        if tuned:
+            for prec in (F64, F32):
+                for n in (1, 2):
+                    mdwf.mdwf_set_tuning(h, prec, n, 128 // Ls)
         bd = torch.from_numpy(b).cuda()
-        x = torch.zeros_like(bd)
-        st, info = mdwf.mdwf_cgne(h, x, bd, nrhs=2, mf_per_rhs=[0.01, 0.05], tol=1e-10, inner_prec=F32)
-        assert st == 0 and all(i.true_res <= 1e-10 for i in info), [i.as_dict() for i in info]
+        for inner in (F32, F64):
+            x = torch.zeros_like(bd)
+            st, info = mdwf.mdwf_cgne(h, x, bd, nrhs=2, mf_per_rhs=[0.01, 0.05], tol=1e-10, inner_prec=inner)
+            assert st == 0 and all(i.true_res <= 1e-10 for i in info), [i.as_dict() for i in info]
+            xs[inner] = x.cpu().numpy()
         phi = torch.from_numpy(np.ascontiguousarray(oracle.split(b[0], dims)[1])).cuda()
         G = torch.empty(U.shape, dtype=torch.complex128, device="cuda")
         S, db5, dc5, st, finfo = mdwf.mdwf_force(h, G, phi, tol=1e-11)
         assert st == 0
     finally:
         mdwf.mdwf_destroy(h)
-    xs = x.cpu().numpy()
-    for r, m in enumerate((0.01, 0.05)):
+    for inner, r, m in ((i, r, m) for i in xs for r, m in enumerate((0.01, 0.05))):
         p = oracle.Params(dims, Ls, 1.8, 1.5, 0.5, m)
-        res = b[r] - oracle.ddw(xs[r], U, p)
-        assert np.linalg.norm(res) / np.linalg.norm(b[r]) <= 1e-7, (Ls, r)
+        res = b[r] - oracle.ddw(xs[inner][r], U, p)
+        assert np.linalg.norm(res) / np.linalg.norm(b[r]) <= 1e-7, (Ls, inner, r)
 
 # t-slab stages, two slabs
 dims, Ls = (4, 4, 4, 8), 8

@@ -34,6 +34,7 @@ def check(got, ref, prec):
     assert (el2 <= 3e-3) if prec == F16N else (emax <= TOL[prec]), (prec, emax, el2)
 
 for dims, Ls, prof in (((4, 4, 4, 4), 8, None), ((4, 4, 2, 4), 16, None),
+                       ((8, 8, 4, 8), 10, None),  # FP64 with two threads a column
                        ((4, 4, 2, 4), 8, ([1.2, 1.9, 1.4, 2.3, 1.1, 1.7, 1.3, 2.0],
                                           [0.1, 0.8, 0.2, 1.0, 0.3, 0.6, 0.4, 0.9]))):
     U = sy.gauge_field(dims, 0.3, 1101)
@@ -44,16 +45,21 @@ for dims, Ls, prof in (((4, 4, 4, 4), 8, None), ((4, 4, 2, 4), 16, None),
     with Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.02, U) as c:
         if prof:
             mdwf.mdwf_set_s_coefficients(c.h, *prof)
-        for prec in (F64, F32, F16N):
-            for dagger in (False, True):
-                check(c.apply(odd, prec, dagger)[0], oracle.m(odd, U, p, dagger=dagger), prec)
+        for dagger in (False, True):
+            ref = oracle.m(odd, U, p, dagger=dagger)
+            for prec in (F64, F32, F16N):
+                for sites in (0, 128 // Ls):  # several threads a column, and the ordinary form
+                    mdwf.mdwf_set_tuning(c.h, prec, 1, sites)
+                    check(c.apply(odd, prec, dagger)[0], ref, prec)
     b = sy.gaussian_field(dims, Ls, 2102)
     h = mdwf.mdwf_create(dims, Ls, 1.8, 1.5, 0.5, 0.02)
     try:
         mdwf.mdwf_load_gauge(h, torch.from_numpy(U).cuda())
         if prof:
             mdwf.mdwf_set_s_coefficients(h, *prof)
-        for inner in (F64, F32, F16N):
+        for inner, sites in ((F64, 0), (F32, 0), (F16N, 0), (F64, 128 // Ls), (F32, 128 // Ls)):
+            for prec in (F64, F32):
+                mdwf.mdwf_set_tuning(h, prec, 1, sites)
             bb = torch.from_numpy(b).cuda()
             x = torch.zeros_like(bb)
             st, info = mdwf.mdwf_cgne(h, x, bb, tol=1e-10, inner_prec=inner)

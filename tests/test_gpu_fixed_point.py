@@ -17,48 +17,89 @@ F64 = mdwf.MDWF_F64
 DIMS, LS = (4, 6, 2, 4), 6
 
 
-def setup(seed=1):
-    U = sy.gauge_field(DIMS, 0.7, 1400 + seed)
-    odd = oracle.split(sy.gaussian_field(DIMS, LS, 2400 + seed), DIMS)[1]
-    return U, odd, oracle.Params(DIMS, LS, 1.8, 1.5, 0.5, 0.02)
+# the FP64 kernels: four threads a column, two, and one (a tuned number of sites selects it)
+FORMS = [((4, 6, 2, 4), 6, 0), ((8, 8, 4, 8), 10, 0), ((4, 6, 2, 4), 6, 21)]
+forms = pytest.mark.parametrize("dims,Ls,sites", FORMS, ids=["four", "two", "one"])
 
 
+def setup(dims, Ls, seed=1):
+    U = sy.gauge_field(dims, 0.7, 1400 + seed)
+    odd = oracle.split(sy.gaussian_field(dims, Ls, 2400 + seed), dims)[1]
+    return U, odd, oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02)
+
+
+def ctx(dims, Ls, sites, U):
+    c = Ctx(dims, Ls, 1.8, 1.5, 0.5, 0.02, U)
+    mdwf.mdwf_set_tuning(c.h, F64, 1, sites)
+    return c
+
+
+@forms
+@pytest.mark.parametrize("dagger", [False, True])
+def test_error_in_the_norm(dims, Ls, sites, dagger):
+    """Gaussian fields: M is 1.2e-16 from long double, the oracle's FP64 1.6e-16: 2e-16 apart, and 4e-16 a bit more."""
+    U, odd, p = setup(dims, Ls, 7)
+    with ctx(dims, Ls, sites, U) as c:
+        _, el2 = rel_err(c.apply(odd, F64, dagger)[0], oracle.m(odd, U, p, dagger=dagger))
+    assert el2 <= 4e-16, el2
+
+
+def largest_within_two_hops(odd, dims):
+    """For each odd site the largest element of odd among the odd sites that reach it through M."""
+    mask = oracle.parity_mask(dims)
+    f = np.zeros(mask.shape)
+    f[mask == 1] = np.abs(odd).max(axis=(0, 2, 3))
+    for _ in range(2):
+        f = np.max([f] + [np.roll(f, d, a) for a in range(4) for d in (1, -1)], axis=0)
+    return f[mask == 1]
+
+
+@forms
 @pytest.mark.parametrize("dagger", [False, True])
 @pytest.mark.parametrize("what", ["sites", "slices", "links"])
-def test_exponents_far_apart(what, dagger):
-    """Magnitudes spread over many decades between sites, slices or links. The result is within 1e-12 of the
-    largest element as everywhere, and each site within 1e-12 of the largest input that reaches it in M: for
-    "sites" that is the largest of its two-hop neighbourhood, so the bound is checked on the whole field only."""
-    U, odd, p = setup()
+def test_exponents_far_apart(what, dims, Ls, sites, dagger):
+    """Magnitudes spread over many decades between sites, slices or links: within 1e-12 of the largest element as
+    everywhere, and (sites, slices) each site within 2e-13 of the largest input that reaches it. A hop adds 8 x 6
+    products whose sizes sum to at most 28 times the largest neighbour, the s-operators at most double a column, so
+    M's terms sum to 0.25 x 28 x 28 x 2 = 400 times the input, and each of the two hops rounds them about twice:
+    1600 x 2^-53."""
+    U, odd, p = setup(dims, Ls)
     rng = np.random.default_rng(5)
     if what == "sites":
         odd = odd * np.exp(8 * rng.standard_normal(odd.shape[1]))[None, :, None, None]
     elif what == "slices":
-        odd = odd * np.exp(-3.0 * np.arange(LS))[:, None, None, None]
+        odd = odd * np.exp(-3.0 * np.arange(Ls))[:, None, None, None]
     else:
         U = U * np.exp(2 * rng.standard_normal(U.shape[:-2]))[..., None, None]
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
-        emax, el2 = rel_err(c.apply(odd, F64, dagger)[0], oracle.m(odd, U, p, dagger=dagger))
+    ref = oracle.m(odd, U, p, dagger=dagger)
+    with ctx(dims, Ls, sites, U) as c:
+        got = c.apply(odd, F64, dagger)[0]
+    emax, el2 = rel_err(got, ref)
     assert emax <= 1e-12 and el2 <= 1e-12, (emax, el2)
+    if what != "links":
+        err = np.abs(got - ref).max(axis=(0, 2, 3))
+        assert (err <= 2e-13 * largest_within_two_hops(odd, dims)).all()
 
 
+@forms
 @pytest.mark.parametrize("k", [-950, -700, 700, 950])
-def test_powers_of_two_commute(k):
+def test_powers_of_two_commute(k, dims, Ls, sites):
     """M(2^k psi) = 2^k M psi to the last bit while nothing under- or overflows: the exponents carry the scale."""
-    U, odd, _ = setup(2)
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+    U, odd, _ = setup(dims, Ls, 2)
+    with ctx(dims, Ls, sites, U) as c:
         one = c.apply(odd, F64)[0]
         two = c.apply(odd * 2.0 ** k, F64)[0]
     assert np.array_equal(two, one * 2.0 ** k)
 
 
+@forms
 @pytest.mark.parametrize("scale", [2.0 ** -1060, 2.0 ** 1010])
-def test_ends_of_the_range(scale):
+def test_ends_of_the_range(scale, dims, Ls, sites):
     """Subnormal fields keep the accuracy that subnormals have (2^-1074 a rounding, under 400 of them a site);
     large ones stay finite."""
-    U, odd, p = setup(3)
+    U, odd, p = setup(dims, Ls, 3)
     psi = odd * scale
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+    with ctx(dims, Ls, sites, U) as c:
         got = c.apply(psi, F64)[0]
     ref = oracle.m(odd, U, p)
     assert np.isfinite(got).all()
@@ -67,27 +108,29 @@ def test_ends_of_the_range(scale):
     assert np.abs(got.view(np.float64) / scale - ref.view(np.float64)).max() <= bound
 
 
-def test_zero_field_and_zero_links():
-    U, odd, p = setup(4)
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+@forms
+def test_zero_field_and_zero_links(dims, Ls, sites):
+    U, odd, p = setup(dims, Ls, 4)
+    with ctx(dims, Ls, sites, U) as c:
         assert not c.apply(np.zeros_like(odd), F64)[0].any()
     U = U.copy()
     U[1] = 0
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+    with ctx(dims, Ls, sites, U) as c:
         emax, _ = rel_err(c.apply(odd, F64)[0], oracle.m(odd, U, p))
     assert emax <= 1e-12
 
 
+@pytest.mark.parametrize("dims,Ls,sites", [((8, 4, 4, 8), 6, 0), ((8, 8, 4, 8), 10, 0), ((8, 4, 4, 8), 6, 21)],
+                         ids=["four", "two", "one"])
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("where", ["field", "link"])
-def test_nonfinite_spreads_as_in_fp64(where, bad):
+def test_nonfinite_spreads_as_in_fp64(where, bad, dims, Ls, sites):
     """A non-finite entry makes the same sites non-finite as FP64 arithmetic (the oracle) does and leaves the
     others as they are without it."""
-    dims = (8, 4, 4, 8)
     U = sy.gauge_field(dims, 0.3, 1405)
-    odd = oracle.split(sy.gaussian_field(dims, LS, 2405), dims)[1]
-    p = oracle.Params(dims, LS, 1.8, 1.5, 0.5, 0.02)
-    with Ctx(dims, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+    odd = oracle.split(sy.gaussian_field(dims, Ls, 2405), dims)[1]
+    p = oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02)
+    with ctx(dims, Ls, sites, U) as c:
         clean = c.apply(odd, F64)[0]
     if where == "field":
         odd = odd.copy()
@@ -95,7 +138,7 @@ def test_nonfinite_spreads_as_in_fp64(where, bad):
     else:
         U = U.copy()
         U[3, 1, 2, 5, 1, 0, 2] = bad
-    with Ctx(dims, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+    with ctx(dims, Ls, sites, U) as c:
         got = c.apply(odd, F64)[0]
     ref = oracle.m(odd, U, p)
     hit = ~np.isfinite(got).all(axis=(0, 2, 3))
@@ -104,12 +147,13 @@ def test_nonfinite_spreads_as_in_fp64(where, bad):
     assert np.array_equal(got[:, ~hit], clean[:, ~hit])
 
 
+@forms
 @pytest.mark.parametrize("mu", [-10.0, -0.3, 3.0, 10.0])
 @pytest.mark.parametrize("dagger", [False, True])
-def test_time_factors(mu, dagger):
-    U, odd, _ = setup(6)
-    p = oracle.Params(DIMS, LS, 1.8, 1.5, 0.5, 0.02, mu=mu)
-    with Ctx(DIMS, LS, 1.8, 1.5, 0.5, 0.02, U) as c:
+def test_time_factors(mu, dims, Ls, sites, dagger):
+    U, odd, _ = setup(dims, Ls, 6)
+    p = oracle.Params(dims, Ls, 1.8, 1.5, 0.5, 0.02, mu=mu)
+    with ctx(dims, Ls, sites, U) as c:
         mdwf.mdwf_set_chemical_potential(c.h, mu)
         emax, _ = rel_err(c.apply(odd, F64, dagger)[0], oracle.m(odd, U, p, dagger=dagger))
     assert emax <= 1e-12
