@@ -268,8 +268,8 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
             return st;
         if ((st = cuda_status(cudaMalloc(&c->mass64, 2 * kMaxRhs * sizeof(double))))) return st;
         if ((st = cuda_status(cudaMalloc(&c->mass32, 2 * kMaxRhs * sizeof(float))))) return st;
-        if ((st = cuda_status(cudaMallocHost(&c->tab_host, total * (sizeof(double) + sizeof(float)) + 2 * kMaxRhs * 12 + 16))))
-            return st;
+        const size_t host = total * (sizeof(double) + sizeof(float)) + 2 * kMaxRhs * 12 + 16;
+        if ((st = cuda_status(cudaMallocHost(&c->tab_host, host)))) return st;
         c->tab_cap = nrhs;
     }
     // host layout: [op][rhs][chir][s'][s]
@@ -299,10 +299,9 @@ int ensure_tables(mdwf_ctx* c, int nrhs, const double* mf_per_rhs) {
         return st;
     if ((st = cuda_status(cudaMemcpyAsync(c->tab32, h32, total * sizeof(float), cudaMemcpyHostToDevice, c->stream))))
         return st;
-    if ((st = cuda_status(cudaMemcpyAsync(c->mass64, hm64, 2 * kMaxRhs * sizeof(double), cudaMemcpyHostToDevice, c->stream))))
-        return st;
-    if ((st = cuda_status(cudaMemcpyAsync(c->mass32, hm32, 2 * kMaxRhs * sizeof(float), cudaMemcpyHostToDevice, c->stream))))
-        return st;
+    const size_t mb64 = 2 * kMaxRhs * sizeof(double), mb32 = 2 * kMaxRhs * sizeof(float);
+    if ((st = cuda_status(cudaMemcpyAsync(c->mass64, hm64, mb64, cudaMemcpyHostToDevice, c->stream)))) return st;
+    if ((st = cuda_status(cudaMemcpyAsync(c->mass32, hm32, mb32, cudaMemcpyHostToDevice, c->stream)))) return st;
     if ((st = cuda_status(cudaStreamSynchronize(c->stream)))) return st;
     memcpy(c->tab_masses, masses, sizeof(double) * nrhs);
     c->tab_nrhs = nrhs;
@@ -350,7 +349,8 @@ int apply_chain(mdwf_ctx* c, void* out, const void* in, int prec, int nrhs, int 
     h.dagger = dagger;
     // z_e = K H_eo w_o, or K^dag H'_eo v_o
     h.mass = mass;
-    h.out = z; h.in = w; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0; h.in_exp = wexp; h.out_exp = zexp;
+    h.out = z; h.in = w; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0;
+    h.in_exp = wexp; h.out_exp = zexp;
     set_sop(c, prec, SOP_K, dagger, h);
     offset_rhs(c, prec, rhs0, h);
     if ((st = launch_hop(c, prec, h))) return st;
@@ -637,8 +637,8 @@ int mdwf_load_gauge(mdwf_ctx* c, const double* U, int where) {
     if (!c->gauge[0]) {
         // the FP64 and FP32 copies and the fixed-point copy that the FP64 hops read: one allocation (each takes a
         // quarter of a millisecond, beside 2 ms for a context). T-slabs have no third copy. Where it would take the
-        // room that the rest of an application needs (four FP64 fields), only its exponents are there, all raw: the FP64
-        // hops then run in FP64 arithmetic.
+        // room that the rest of an application needs (four FP64 fields), only its exponents are there, all raw: the
+        // FP64 hops then run in FP64 arithmetic.
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t b64 = up(nlink * link_store_bytes(MDWF_F64)), b32 = up(nlink * link_store_bytes(MDWF_F32));
         const size_t bexp = c->slab ? 0 : up(nlink * sizeof(int));

@@ -106,7 +106,8 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const double* part, in
 // Column-blocked update for the fused iteration: block = (Ls, SB) threads
 // covering SB whole s-columns. x += alpha p; p = r + beta p; then
 // w = M_phi p = b5 p_s + c5 (P+ p_{s-1} + P- p_{s+1}) (mass -m on the
-// wrap-around; without its factor b5 where the operators leave theirs out, sop_scale) with the new p of the neighbouring slices taken from shared
+// wrap-around; without its factor b5 where the operators leave theirs out,
+// sop_scale) with the new p of the neighbouring slices taken from shared
 // memory, so that the first hop of the next iteration reads w without
 // gathering along s. With per-slice coefficients gs holds the gather factors
 // of row s, [gown][gfac][gscale] (64 each): b5(s) = gscale gown and
@@ -439,8 +440,8 @@ static int launch_pupd_w(Solver& S, void* x, void* r, void* p, void* w) {
     LaunchScope scope(c, KB_BLAS * 3 + PP, S.n5() * (3.0 * site_bytes(PR) + 3.0 * site_bytes(PP)), S.n5() * 144.0);
     if (cudaError_t e = launch_pdl(k_pupd_w<PR, PR, PP>, grid, block, smem, c->stream, make_field<PR>(x, S.g, S.nrhs),
                                    make_field<PR>(r, S.g, S.nrhs), make_field<PP>(p, S.g, S.nrhs),
-                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5 / phi, c->c5 / phi,
-                                   fx_exp_if(c, PP, w, S.nrhs)))
+                                   make_field<PP>(w, S.g, S.nrhs), (const double*)S.sc, mass, gs, S.g, c->b5 / phi,
+                                   c->c5 / phi, fx_exp_if(c, PP, w, S.nrhs)))
         return cuda_status(e);
     return check_launch();
 }
@@ -499,7 +500,8 @@ static int cg_iteration_fused(Solver& S, void* x, void* r, void* p, void* t, voi
     h.mat2 = nullptr;
     h.no_t = 0;
     // K1' does not need alpha, so alpha is formed after it is launched, beside its end
-    h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0; h.dagger = 1;
+    h.out = c->tmp[0].p; h.in = c->tmp[1].p; h.x = nullptr; h.coef = 1.0; h.unscaled = 1; h.out_parity = 0;
+    h.dagger = 1;
     h.in_exp = vexp; h.out_exp = zexp;
     set_sop(c, PP, SOP_K, 1, h);
     h.fuse = 0;
@@ -1149,7 +1151,8 @@ extern "C" int mdwf_cgne(mdwf_ctx* c, double* x, const double* b, int nrhs, cons
         size_t free_b = 0, total_b = 0;
         if ((st = cuda_status(cudaMemGetInfo(&free_b, &total_b)))) return st;
         auto grow = [](size_t need_b, const Workspace& ws) { return need_b > ws.bytes ? need_b - ws.bytes : 0; };
-        size_t extra = grow(keep_need, c->io) + grow(fx_field_bytes(g, nrhs), c->tmp[0]) + grow(fx_field_bytes(g, nrhs), c->tmp[1]);
+        const size_t fxn = fx_field_bytes(g, nrhs);
+        size_t extra = grow(keep_need, c->io) + grow(fxn, c->tmp[0]) + grow(fxn, c->tmp[1]);
         // the solver workspace, or the autotuner's two scratch fields before it (freed after tuning)
         size_t later = grow(
             solver_bytes(c, nrhs, prm.inner_prec, red_blocks(nrhs), hop_blocks(c, prm.inner_prec, nrhs)), c->solver);

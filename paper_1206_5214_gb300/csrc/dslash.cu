@@ -9,12 +9,13 @@ namespace mdwf {
 
 template <int P> int launch_hop_t(mdwf_ctx* c, const HopLaunch& h);
 
-// The block shape of a hop launch: as many whole s-columns as fit 128 threads, or the autotuned number. Where such blocks
-// are so few that the time of a hop is that of one thread's chain of eight neighbours, four or (FP64) two threads share a
-// column (STAGE 5 and 6 of the kernel) and a block holds a fourth or half of the columns. M alone in us, one, two and four
-// threads a column, by the number of ordinary blocks on 152 SMs:
+// The block shape of a hop launch: as many whole s-columns as fit 128 threads, or the autotuned number. Where such
+// blocks are so few that the time of a hop is that of one thread's chain of eight neighbours, four or (FP64) two
+// threads share a column (STAGE 5 and 6 of the kernel) and a block holds a fourth or half of the columns. M alone in
+// us, one, two and four threads a column, by the number of ordinary blocks on 152 SMs:
 //   FP32: 8 blocks 16.4, -, 13.7; 128 blocks 17.0, -, 14.4; 140 blocks 20.5, -, 16.5; 256 blocks 16.5, -, 20.5
-//   FP64: 8 blocks 47, 34, 30; 64 blocks 49, 34, 34; 128 blocks 49, 43, 56; 205 blocks 64, 46, 72; 256 blocks 64, 77, 95
+//   FP64: 8 blocks 47, 34, 30; 64 blocks 49, 34, 34; 128 blocks 49, 43, 56; 205 blocks 64, 46, 72;
+//         256 blocks 64, 77, 95
 // FP32 gains while the ordinary form leaves an SM at most one block. The FP64 split forms run three blocks per SM:
 // two threads a column pay while those blocks are one wave (205 blocks make 410, 256 make 512, of 456), four while
 // the integer pipe is not the limit.

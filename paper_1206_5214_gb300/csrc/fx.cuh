@@ -19,10 +19,10 @@
 // eight neighbours' components, times a link entry of one, is 2^54 to 2^55 units. FP64 arithmetic rounds every
 // partial sum to 2^-53 of its size. M and M^dag against long double, 24 cases of lattices, Ls, links and
 // coefficients and four kinds of input (Gaussian, slices falling by e^-2, point source, sites spread over decades):
-// mean relative error 1.62e-16 with FP64 hops, 1.26e-16 with these (and 1.15e-16 with the s-operators as they are
-// now); per site as well. Ranges: a neighbour's projected component is below 2^59 (limbs |hi| <= 2^27, |lo| <=
-// 2^31), so the middle sum is at most 6 (2^29 2^31 + 2^31 2^27) = 7.5 2^60 < 2^63, a transported component at most
-// 6 2^56, and the sum of eight terms at most 48 2^56 < 2^63.
+// mean relative error 1.62e-16 with FP64 hops, 1.18e-16 with these and today's s-operators; per site as well.
+// Ranges: a neighbour's projected component is below 2^59 (limbs |hi| <= 2^27, |lo| <= 2^31), so the middle sum is
+// at most 6 (2^29 2^31 + 2^31 2^27) = 7.5 2^60 < 2^63, a transported component at most 6 2^56, and the sum of eight
+// terms at most 48 2^56 < 2^63.
 //
 // Small parts beside large ones: the error above is relative to the largest component that reaches a site, where
 // FP64 arithmetic errs relative to what each component is made of. The two differ where parts of the field do not

@@ -35,8 +35,8 @@ __device__ __forceinline__ void fx_colour(const int4* u, int si, int sj, const l
 #pragma unroll
         for (int j = 0; j < 3; ++j) r[j] = __ldg(u + i * si + j * sj);
         const long long half = 0x80000000ll;  // half of the place that is kept
-        // four sums (2 spins, re and im) side by side, since one sum's multiply-adds depend on each other (two at a time:
-        // M 1.021 against 1.004 ms; the upper parts beside them: 1.052, registers)
+        // four sums (2 spins, re and im) side by side, since one sum's multiply-adds depend on each other (two at a
+        // time: M 1.021 against 1.004 ms; the upper parts beside them: 1.052, registers)
         long long m[4] = {half, half, half, half};
 #pragma unroll
         for (int j = 0; j < 3; ++j)
@@ -47,7 +47,8 @@ __device__ __forceinline__ void fx_colour(const int4* u, int si, int sj, const l
                     const int k = 6 * a + 2 * j, n = 3 * a + j;
                     const int u = p == 0 ? r[j].y : p == 1 ? r[j].x : p == 2 ? r[j].w : r[j].z;
                     m[2 * a] = mad_wide(u, p == 0 ? hl[k] : p == 1 ? hh[k] : p == 2 ? nl[n] : nh[n], m[2 * a]);
-                    m[2 * a + 1] = mad_wide(u, p == 0 ? hl[k + 1] : p == 1 ? hh[k + 1] : p == 2 ? hl[k] : hh[k], m[2 * a + 1]);
+                    m[2 * a + 1] =
+                        mad_wide(u, p == 0 ? hl[k + 1] : p == 1 ? hh[k + 1] : p == 2 ? hl[k] : hh[k], m[2 * a + 1]);
                 }
 #pragma unroll
         for (int k = 0; k < 4; ++k) m[k] >>= 32;

@@ -367,7 +367,6 @@ constexpr int kPrefetchMinBlocks = 7;
 // threads per (site, s) of a STAGE
 constexpr int split_of(int stage) { return stage == 5 ? 4 : stage == 6 ? 2 : 1; }
 
-
 template <int T> struct TermOf {
     static constexpr int MU = T / 2;
     static constexpr bool FWD = T % 2 == 0;
@@ -691,14 +690,16 @@ constexpr bool kShuffleBidiag = MDWF_SHUFFLE_BIDIAG != 0;
 #endif
 
 // STAGE: 0 neighbour spinors loaded into registers, 1 staged per thread with
-// cp.async, 2 whole neighbour columns copied by the copy engine (bulk).
+// cp.async, 2 whole neighbour columns copied by the copy engine (bulk), 3 the
+// next neighbour prefetched into a second register buffer, 5 and 6 below.
 // LSR: Ls fixed at compile time for the epilogue's register-held columns (the
 // launcher picks it when Ls matches), or -1 for the run-time choice; one
 // fixed length leaves the other lengths' code and its register demand out of
 // the kernel.
 // STAGE 5: a fourth of the thread block's columns, four threads (threadIdx.z = mu) per (site, s): each takes the two
-// terms of its direction, and their sums meet in shared memory. STAGE 6 (FP64): two threads with four terms each. For lattices whose columns leave the SMs
-// with one block or less, where a hop takes as long as one thread's chain of eight neighbours (hop_shape).
+// terms of its direction, and their sums meet in shared memory. STAGE 6 (FP64): half of the columns, two threads with
+// four terms each. For lattices whose columns leave the SMs with one block or less, where a hop takes as long as one
+// thread's chain of eight neighbours (hop_shape).
 template <int P, bool DAG, bool XPAY, int FUSE, int STAGE, int LSR, bool DD = false>
 __global__ void __launch_bounds__(128, STAGE == 1   ? MDWF_MINB_STAGE
                                       : STAGE >= 5 ? (P == MDWF_F64 ? 3 : 4)
@@ -1069,14 +1070,15 @@ static int launch_hop_variant(mdwf_ctx* c, const HopLaunch& h, const HopParams<t
         if (!hp.chem) fx.xf = fx.xb = 0;
     }
     LaunchScope scope(c, base * 3 + P, bytes, flops);
-    if (cudaError_t e = launch_pdl(kern, grid, block, smem, c->stream, out, in, xf, U, hp, fa, fx)) return cuda_status(e);
+    if (cudaError_t e = launch_pdl(kern, grid, block, smem, c->stream, out, in, xf, U, hp, fa, fx))
+        return cuda_status(e);
     return check_launch();
 }
 
 // Load strategy per launch (mdwf_set_staging). The FP32 and FP16 operators
-// without the input gather have the staged variants; by default (mode 0, and
-// mode 3) they prefetch the next neighbour into registers. Mode 4 uses the
-// plain loads everywhere.
+// have the staged variants; by default (mode 0, and mode 3) they prefetch the
+// next neighbour into registers, and on the smallest lattices mode 0 takes the
+// split forms of hop_shape. Mode 4 uses the plain loads everywhere.
 template <int P, bool D, bool X, int FU>
 static int launch_hop_pick(mdwf_ctx* c, const HopLaunch& h, const HopParams<typename PrecTraits<P>::real>& hp) {
     if constexpr (FU == FUSE_NONE && P != MDWF_F16N) {
@@ -1158,8 +1160,10 @@ int launch_hop_t(mdwf_ctx* c, const HopLaunch& h) {
         return MDWF_EINVAL;
     }
     if (h.dagger)
-        return X ? launch_hop_pick<P, true, true, FUSE_NONE>(c, h, hp) : launch_hop_pick<P, true, false, FUSE_NONE>(c, h, hp);
-    return X ? launch_hop_pick<P, false, true, FUSE_NONE>(c, h, hp) : launch_hop_pick<P, false, false, FUSE_NONE>(c, h, hp);
+        return X ? launch_hop_pick<P, true, true, FUSE_NONE>(c, h, hp)
+                 : launch_hop_pick<P, true, false, FUSE_NONE>(c, h, hp);
+    return X ? launch_hop_pick<P, false, true, FUSE_NONE>(c, h, hp)
+             : launch_hop_pick<P, false, false, FUSE_NONE>(c, h, hp);
 }
 
 }  // namespace mdwf

@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(kPackLinks) gauge_pack_kernel(double2* u64, fl
         swapped[tid] = (x + y + z + (int)q) & 1;
     }
     __syncthreads();
-    // link r of the block in the order of the copies, r = (parity 4 + mu) sites / 2 + k: its place in the tile and there
+    // link r of the block in the order of the copies, r = (parity 4 + mu) sites / 2 + k: its places in the tile and
+    // there
     const int half = sites / 2;
     auto place = [&](int r) {
         const int q = r / half, k = r % half;

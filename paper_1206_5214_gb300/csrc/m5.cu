@@ -21,10 +21,11 @@ __device__ __forceinline__ void store_m5(const Field<P>& f, int* exp, long long 
 }
 
 // FORM: the operators that read a spinor and its two neighbours straight from memory (below), whole columns in
-// shared memory, or dense tables. Blocks per SM: FP32 and FP16+norm eight (64 registers; at 75 and six blocks M_phi
-// of 16^3 x 32 x 16 took 31.0 and 26.6 us, now 29.8 and 24.6). FP64 direct four, 71 us (six: 105); FP64 columns,
-// which wait for the FP64 pipe and for each other, six: A^dag 144 us at 80 registers with some spilled, 152 with
-// five, 176 with four, and 162 with four and no rule on the parts of a spinor (fx.cuh); FP64 dense four.
+// shared memory, or dense tables: kernels of their own, since in one the registers of each form held the others back.
+// Blocks per SM: FP32 and FP16+norm eight (64 registers; at 75 and six blocks M_phi of 16^3 x 32 x 16 took 31.0 and
+// 26.6 us, now 30.5 and 24.5). FP64 direct four, 72 us (six in one kernel: 105); FP64 columns, which wait for the FP64
+// pipe and for each other, six: A^dag 142 us at 78 registers (one kernel with four blocks, 120 registers: 176); FP64
+// dense four.
 enum { M5_DIRECT, M5_COLUMNS, M5_DENSE };
 template <int P, bool XPAY, int FORM>
 __global__ void __launch_bounds__(128, P != MDWF_F64 ? 8 : FORM == M5_COLUMNS ? 6 : 4)

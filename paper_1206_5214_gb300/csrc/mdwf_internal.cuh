@@ -808,7 +808,7 @@ struct mdwf_ctx {
     bool dense_s = false;
     bool dense_s_base = false;  // the choice for constant coefficients
     // per-slice coefficients b5(s), c5(s) (Sec. 2.1, Sec. 4.3); when set, every s-operator
-    // is a dense table and the gather of the hop takes per-slice factors from
+    // is a dense table and the CG's vector update takes per-slice factors of M_phi from
     // gs64 / gs32 = [gown(s)][gfac(s)][gscale(s)], 64 entries each
     bool sdep = false;
     // chemical potential on the time links (0: none)
